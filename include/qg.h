@@ -206,11 +206,12 @@ int qg_eval_grad(qg_ctx *h, const void *x, double *obj, void *g);
  * (for example code running under an allocator lock, inside a host callback, or in a process
  * whose memory pool is already sized and frozen).  The paper has no counterpart: it is an
  * interface addition.  The handle's set-up data (made by qg_create) is reused; every
- * per-evaluation work buffer comes from one file-scope static device array of 16 MiB that every
- * GPU loading the library holds from load until the process exits.  The caller passes the inputs
+ * per-evaluation work buffer comes from one file-scope static device array of 32 MiB (16 MiB of work
+ * buffers, and at most as much for the hot rows' sums of stage 2) that every GPU loading the library
+ * holds from load until the process exits.  The caller passes the inputs
  * and outputs: x (device, qg_num_vars elements), obj (device, n_inst doubles) and g (device,
  * qg_num_vars elements, required).  Results equal those of qg_eval_grad.
- *  - Handles whose work buffers need more than 16 MiB (e.g. large batches) are rejected with
+ *  - Handles whose work buffers need more than 16 MiB without those sums (e.g. large batches) are rejected with
  *    QG_ERR_UNSUPPORTED and a message giving the size needed; so are handles on the sparse DC
  *    solver (QG_DC_SPARSE), whose solve buffers are not carved from the array, and handles with
  *    contingency screening (0 < ctg_frac < 1), whose compacted line-outage block is not either.

@@ -568,7 +568,7 @@ std::vector<df32> to_dc<df32>(const std::vector<double> &v) {
 
 // A stage holds at most three spans per instance (stage 1: DC flows, branches, zones) plus one
 // for the sparse solver's adjoint right-hand side, so MAXB instances never overflow the table.
-static_assert(MAXSPAN >= 3 * MAXB + 1, "span table too small for MAXB instances");
+static_assert(MAXSPAN >= 4 * MAXB + 1, "span table too small for MAXB instances");
 
 void add_span(Spans &S, int per_t, int nt, int inst, int role) {
   if (per_t <= 0 || nt <= 0) return;
@@ -583,6 +583,13 @@ void add_span(Spans &S, int per_t, int nt, int inst, int role) {
 
 int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 
+// Elements of the hot rows' column partials (Dev::pkh) over the batch.
+long long hot_elems(const Plan &P) {
+  long long n = 0;
+  for (int b = 0; b < P.tab.n_inst; ++b) n += (long long)P.tab.I[b].hot * P.tab.I[b].T * P.tab.I[b].Kp;
+  return n;
+}
+
 // Instance table, spans of the five stage kernels and objective-slot owners.
 int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
   Plan &P = h->plan;
@@ -590,7 +597,7 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
   std::memset(&P, 0, sizeof(P));
   P.tab.n_inst = B;
   long long x0 = 0, tb0 = 0, tm0 = 0, tg0 = 0, tz0 = 0, tk0 = 0, pg0 = 0, l0 = 0, pm0 = 0, pk0 = 0, gi0 = 0, tx0 = 0,
-            pf0 = 0, lm0 = 0, rm0 = 0;
+            pf0 = 0, lm0 = 0, rm0 = 0, ph0 = 0;
   int xf0 = 0;
   // Contingency block shape, shared by the batch: about one wave of CTG_WAVE blocks when the
   // 64 x 64 tiles are few (the periods split across blocks), several waves when they are many
@@ -633,6 +640,13 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
   const int cb = h->opt.ctg_bound;
   const int ctg_lazy = cb == QG_CTG_BOUND_LAZY || (cb == QG_CTG_BOUND_AUTO && el_all > 0 && 2 * el_large >= el_all);
   const int ctg_bound = ctg_lazy || cb == QG_CTG_BOUND_EAGER;
+  // Stage 2 evaluates hot rows (over their limit before any outage) on their own where that pays: on
+  // plans whose elements are mostly large grids' (day-ahead grid, 440 hot rows of 35,000 per period: stage 2
+  // 1.85 -> 0.62 ms on the mixed path, 19.3 -> 4.4 ms on the FP64 path), and on the FP64 path above
+  // SMALL_PLAN.  On small plans the blocks and stage 3's longer sums cost what they save: rt617 FP64, a step
+  // at an iterate without overloads 113 -> 118 us, with 10 hot rows per period 180 -> 157; mixed, stage 2
+  // 16.2 us in the screen, 15.5-20 us with.
+  const bool hot_rows = (el_all > 0 && 2 * el_large >= el_all) || (h->opt.precision == QG_FP64 && bp > SMALL_PLAN);
   P.tab.s3q = small_mixed ? S3_SPLIT_MAX : 1;
   int bus0 = 0, br0 = 0, gen0 = 0, zone0 = 0, ctg0 = 0, gb0 = 0, tp0 = 0, bal0 = 0, adj0 = 0;
   for (int b = 0; b < B; ++b) {
@@ -651,6 +665,16 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
     D.n_mg = ceil_div(D.n_mt, D.ctg_mg);
     D.ctg_tb = ceil_div(H.T, std::min(ntc_all, H.T));
     D.ctg_ntc = ceil_div(H.T, D.ctg_tb);
+    // hot-row blocks of stage 2 (s2_hot): a contingency block's tiles; its periods too on the mixed path
+    // (the objective keeps its order of summation), on the FP64 path so few that the blocks are
+    // several waves
+    D.hot = hot_rows && H.Ks > 0 ? D.n_mg : 0;
+    D.hot_mg = D.ctg_mg;
+    D.hot_tb = D.ctg_tb;
+    if (h->opt.precision == QG_FP64)
+      D.hot_tb = (int)std::max(1LL, std::min((long long)D.ctg_tb, (long long)H.T * D.n_mg * ceil_div(H.Ks, HOT_BK) / (8 * 152)));
+    D.hot_ntc = ceil_div(H.T, D.hot_tb);
+    if (D.hot) P.hot = 1;
     // latency layouts of small plans on the mixed path (see `small` below): four threads per
     // branch-period in stage 3, two CSR packs per warp in stage 4
     D.s4p = small_mixed ? S4_PACKS : 1;
@@ -658,7 +682,7 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
     D.bal0 = bal0; D.n_bal_pack = (int)H.bal_code.size() / PACK;
     D.adj0 = adj0; D.n_adj_pack = (int)H.adj_code.size() / PACK;
     D.x0 = x0; D.tb0 = tb0; D.tm0 = tm0; D.tg0 = tg0; D.tz0 = tz0; D.tk0 = tk0; D.pg0 = pg0; D.l0 = l0;
-    D.pm0 = pm0; D.pk0 = pk0; D.gi0 = gi0; D.pf0 = pf0; D.lm0 = lm0; D.rm0 = rm0;
+    D.pm0 = pm0; D.pk0 = pk0; D.gi0 = gi0; D.pf0 = pf0; D.lm0 = lm0; D.rm0 = rm0; D.ph0 = ph0;
     D.ctg_bound = ctg_bound; D.ctg_lazy = ctg_lazy;
     D.inv_n = 1.0 / H.n;
     D.hours = 0.0;
@@ -673,7 +697,7 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
     rm0 += (long long)H.T * D.n_mt * CT_BM;  // ctg_ntc ceil(ctg_tb / 8) <= T chunks, whatever the shape
     P.ctg_lazy = ctg_lazy;
     P.ctg_bound = ctg_bound;
-    pm0 += (long long)D.n_kt * H.T * H.M; pk0 += (long long)D.n_mg * H.T * H.Ks; gi0 += (long long)H.T * (D.Gc + 1);
+    pm0 += (long long)D.n_kt * H.T * H.M; pk0 += (long long)D.n_mg * H.T * H.Ks; ph0 += (long long)D.hot * H.T * D.Kp; gi0 += (long long)H.T * (D.Gc + 1);
     bus0 += H.n; br0 += H.M; gen0 += H.G; zone0 += H.Z; ctg0 += H.Ks; gb0 += D.Gb; tp0 += H.T;
     bal0 += (int)H.bal_code.size(); adj0 += (int)H.adj_code.size();
     P.maxT = std::max(P.maxT, H.T);
@@ -706,6 +730,7 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
   if (bal1)
     for (int b = 0; b < B; ++b) add_span(P.s1, ceil_div(I[b].n_bal_pack, PACKS_PER_BLOCK), I[b].T, b, R_BUS);
   for (int b = 0; b < B; ++b) add_span(P.s1, I[b].Z, I[b].T, b, R_ZONE);
+  for (int b = 0; b < B; ++b) add_span(P.s2, I[b].hot * I[b].hot_ntc * ceil_div(I[b].K, HOT_BK), I[b].hot > 0 ? 1 : 0, b, R_HOT);
   for (int b = 0; b < B; ++b) add_span(P.s2, I[b].ctg_ntc * I[b].n_mg * I[b].n_kt, I[b].K > 0 ? 1 : 0, b, R_CTG);
   if (!bal1) {
     // a stage-2 bus-balance block is a few microseconds of work: on large plans each covers several
@@ -868,7 +893,7 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
   std::vector<int> br_kidx, gen_bus, gen_zone, gen_gb, gb_ptr{0}, gb_gen, gb_dev0, gb_ndev, zgen_ptr{0}, zgen, ctg_br,
       bal_code, bal_row,
       adj_code, adj_row, br_xf, xf_br;
-  std::vector<double> br_g, br_b, br_hch, br_smax, br_s2, ga, gbv, gcr, gpmax, gramp, load_p, load_q, rreq, dt, lo, hi,
+  std::vector<double> br_g, br_b, br_hch, br_smax, br_s2, br_sctg, ga, gbv, gcr, gpmax, gramp, load_p, load_q, rreq, dt, lo, hi,
       ltot, ptdfg, ptdfaT, cload, rsum, lodf, gsgn, gpmin, gqmin, gqmax, gcon, gcsu, gcsd, guinit, blk_c, blk_lo, blk_w;
   std::vector<int> blk_ptr{0};
   for (int b = 0; b < B; ++b) {
@@ -882,6 +907,7 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
       br_hch.push_back(0.5 * H.bch[j]);
       br_smax.push_back(H.smax[j]);
       br_s2.push_back(H.sctg[j] * H.sctg[j]);
+      br_sctg.push_back(std::sqrt((Real)br_s2.back()));
     }
     for (int j = 0; j < H.Ks; ++j) {
       br_kidx[D.br0 + H.ctg[H.sel[j]]] = j;
@@ -1003,7 +1029,7 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
   UPI(br_kidx, br_kidx) UPI(gen_bus, gen_bus) UPI(gen_zone, gen_zone) UPI(gen_gb, gen_gb) UPI(gb_ptr, gb_ptr)
   UPI(gb_gen, gb_gen) UPI(gb_dev0, gb_dev0) UPI(gb_ndev, gb_ndev) UPI(zgen_ptr, zgen_ptr) UPI(zgen, zgen) UPI(ctg_br, ctg_br) UPI(bal_code, bal_code)
   UPI(bal_row, bal_row) UPI(adj_code, adj_code) UPI(adj_row, adj_row) UPI(br_xf, br_xf) UPI(xf_br, xf_br)
-  UPR(br_g, br_g) UPR(br_b, br_b) UPR(br_hch, br_hch) UPR(br_smax, br_smax) UPR(br_s2ctg, br_s2)
+  UPR(br_g, br_g) UPR(br_b, br_b) UPR(br_hch, br_hch) UPR(br_smax, br_smax) UPR(br_s2ctg, br_s2) UPR(br_sctg, br_sctg)
   UPR(gen_a, ga) UPR(gen_b, gbv) UPR(gen_cr, gcr) UPR(gen_pmax, gpmax)
   UPR(gen_sgn, gsgn) UPR(gen_pmin, gpmin) UPR(gen_qmin, gqmin) UPR(gen_qmax, gqmax) UPR(gen_con, gcon)
   UPR(gen_csu, gcsu) UPR(gen_csd, gcsd) UPR(gen_uinit, guinit) UPI(blk_ptr, blk_ptr) UPR(blk_c, blk_c)
@@ -1092,6 +1118,8 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
     }
     if ((rc = dalloc(h, &pz, (size_t)spk)) || (rc = dalloc(h, &zs, (size_t)stk))) return rc;
     d.pz = pz;
+    if ((rc = dalloc(h, &pz, (size_t)std::max(1LL, hot_elems(P))))) return rc;
+    d.pzh = pz;
     d.zs = zs;
     d.score = 1;
     for (int b = 0; b < B; ++b)
@@ -1159,7 +1187,7 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
   d.n_pairs = sTG;
   WR(pf, sTM) WR(qf, sTM) WR(pt, sTM) WR(qt, sTM) WR(qm2, sTM) WR(fre, sTM) WR(fk, sTK) WR(pold, sTG) WR(uold, sTG)
   WR(dP, sTn) WR(dQ, sTn) WR(dZ, sTZ) WR(pm, sPM) WR(pq, sPM) WR(pk, sPK) WR(gF, sTM) WR(avf, sTM) WR(avo, sTM)
-  WR(ad, sTM) WR(atx, sTX)
+  WR(ad, sTM) WR(atx, sTX) WR(pkh, std::max(1LL, hot_elems(P)))
   WD(gip, sGI)
   WF(f32, sTM) WF(fk32, sTK)
 #undef WR
@@ -1168,6 +1196,8 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
   unsigned char *qs;
   if ((rc = dalloc(h, &qs, (size_t)sTM))) return rc;
   d.qside = qs;
+  if ((rc = dalloc(h, &qs, (size_t)sTM))) return rc;
+  d.hot = qs;
   long long sPF = 0;
   for (int b = 0; b < B; ++b) sPF += (long long)P.tab.I[b].n_kt * P.tab.I[b].T * P.tab.I[b].n_mt;
   unsigned char *pf;
@@ -1292,11 +1322,17 @@ int replan_dev(qg_ctx *h, Dev<Real, Dc> &d, const Knobs &kn) {
   Real *pk;
   if ((rc = dalloc(h, &pk, (size_t)std::max(1LL, spk)))) return rc;
   d.pk = pk;
+  dfree(h, d.pkh);
+  if ((rc = dalloc(h, &pk, (size_t)std::max(1LL, hot_elems(P))))) return rc;
+  d.pkh = pk;
   if (d.score) {
     dfree(h, d.pz);
     Real *pz;
     if ((rc = dalloc(h, &pz, (size_t)std::max(1LL, spk)))) return rc;
     d.pz = pz;
+    dfree(h, d.pzh);
+    if ((rc = dalloc(h, &pz, (size_t)std::max(1LL, hot_elems(P))))) return rc;
+    d.pzh = pz;
   }
   d.n_obj12 = (int)slot_map.size();
   d.n_gen_slots = P.n_gen_slots;
@@ -1307,7 +1343,7 @@ int replan_dev(qg_ctx *h, Dev<Real, Dc> &d, const Knobs &kn) {
   int *si;
   if ((rc = upload(h, &si, slot_map))) return rc;
   d.slot_map = si;
-  const cudaError_t e = prepare_eval<Real, Dc>(P.maxTB, h->screen, P.ctg_lazy != 0);
+  const cudaError_t e = prepare_eval<Real, Dc>(P.maxTB, h->screen, P.ctg_lazy != 0, P.hot != 0);
   if (e != cudaSuccess) {
     cudaGetLastError();  // a refused attribute is not a sticky error
     return fail(h, QG_ERR_UNSUPPORTED, std::string("prepare_eval: ") + cudaGetErrorString(e));
@@ -1418,8 +1454,10 @@ __global__ void k_host_out(const Real *g, double *hg, long long n, const double 
 // cudaGetSymbolAddress, looked up once per device.
 // =============================================================================================
 
-constexpr size_t NOALLOC_SCRATCH_BYTES = size_t(16) << 20;  // 16 MiB
-static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES];
+constexpr size_t NOALLOC_SCRATCH_BYTES = size_t(16) << 20;  // 16 MiB of work buffers, and
+constexpr size_t NOALLOC_HOT_BYTES = size_t(16) << 20;      // the hot rows' column sums and flags: never more
+                                                            // than the work buffers (see carve_hot)
+static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_SCRATCH_BYTES + NOALLOC_HOT_BYTES];
 
 namespace {
 
@@ -1439,7 +1477,7 @@ int noalloc_scratch(qg_ctx *h, unsigned char **out) {
     if (e != cudaSuccess || !ptr)
       return fail(h, QG_ERR_CUDA, std::string("cudaGetSymbolAddress(scratch): ") + cudaGetErrorString(e));
     g_noalloc_ptr[dev] = static_cast<unsigned char *>(ptr);
-    bounds_register(ptr, NOALLOC_SCRATCH_BYTES);
+    bounds_register(ptr, NOALLOC_SCRATCH_BYTES + NOALLOC_HOT_BYTES);
   }
   *out = g_noalloc_ptr[dev];
   return QG_OK;
@@ -1469,7 +1507,7 @@ size_t carve_scratch(const qg_ctx *h, unsigned char *base, size_t cap, Dev<Real,
   d.pf = (Real *)take(R * sTM); d.qf = (Real *)take(R * sTM); d.pt = (Real *)take(R * sTM);
   d.qt = (Real *)take(R * sTM); d.qm2 = (Real *)take(R * sTM); d.fre = (Real *)take(R * sTM);
   d.gF = (Real *)take(R * sTM); d.avf = (Real *)take(R * sTM); d.avo = (Real *)take(R * sTM);
-  d.ad = (Real *)take(R * sTM); d.qside = take(sTM); d.f32 = (float *)take(4 * sTM);
+  d.ad = (Real *)take(R * sTM); d.qside = take(sTM);  d.f32 = (float *)take(4 * sTM);
   d.atx = (Real *)take(R * std::max(1LL, sTX));
   d.fk = (Real *)take(R * sTK); d.fk32 = (float *)take(4 * sTK); d.pold = (Real *)take(R * sTG);
   d.uold = (Real *)take(R * sTG);
@@ -1491,6 +1529,20 @@ size_t carve_scratch(const qg_ctx *h, unsigned char *base, size_t cap, Dev<Real,
   return off;
 }
 
+// Carve the hot rows' flags and column sums out of [base, base + NOALLOC_HOT_BYTES); false if they do
+// not fit.  They take T M bytes and at most n_mg T Kp elements (Kp < K + 4, n_mg <= M / 64 + 1), and the
+// work buffers hold n_mg T K, 2 ceil(K / 64) T M and more than 12 T M elements: a handle whose work
+// buffers fit 16 MiB fits here.
+template <typename Real, typename Dc>
+bool carve_hot(const qg_ctx *h, unsigned char *base, Dev<Real, Dc> &d) {
+  const size_t sums = (sizeof(Real) * (size_t)hot_elems(h->plan) + 255) & ~size_t(255);
+  size_t flags = 0;
+  for (int b = 0; b < h->n_inst; ++b) flags += (size_t)h->plan.tab.I[b].T * h->plan.tab.I[b].M;
+  d.pkh = (Real *)base;
+  d.hot = base + sums;
+  return sums + flags <= NOALLOC_HOT_BYTES;
+}
+
 template <typename Real, typename Dc>
 int eval_noalloc(qg_ctx *h, Dev<Real, Dc> d, const void *x, double *obj, void *g) {
   unsigned char *base = nullptr;
@@ -1501,6 +1553,8 @@ int eval_noalloc(qg_ctx *h, Dev<Real, Dc> d, const void *x, double *obj, void *g
     return fail(h, QG_ERR_UNSUPPORTED, "qg_eval_grad_noalloc: this handle needs " + std::to_string(need) +
                                            " bytes of scratch; the static scratch holds " +
                                            std::to_string(NOALLOC_SCRATCH_BYTES));
+  if (!carve_hot(h, base + NOALLOC_SCRATCH_BYTES, d))
+    return fail(h, QG_ERR_UNSUPPORTED, "qg_eval_grad_noalloc: the hot rows' sums of this handle do not fit the static scratch");
   d.obj = obj;
   d.g = static_cast<Real *>(g);
   d.trace = nullptr;
@@ -1608,8 +1662,8 @@ int qg_create_batch(qg_ctx **out, int32_t n_inst, const qg_network *net, const q
   }
   rc = mixed(h) ? build_device<float, df32>(h, h->d32, slot_map) : build_device<double, double>(h, h->d64, slot_map);
   if (!rc) {
-    cudaError_t e = mixed(h) ? prepare_eval<float, df32>(h->plan.maxTB, h->screen, h->plan.ctg_lazy != 0)
-                             : prepare_eval<double, double>(h->plan.maxTB, h->screen, h->plan.ctg_lazy != 0);
+    cudaError_t e = mixed(h) ? prepare_eval<float, df32>(h->plan.maxTB, h->screen, h->plan.ctg_lazy != 0, h->plan.hot != 0)
+                             : prepare_eval<double, double>(h->plan.maxTB, h->screen, h->plan.ctg_lazy != 0, h->plan.hot != 0);
     if (e != cudaSuccess) rc = fail(h, QG_ERR_UNSUPPORTED, std::string("prepare_eval: ") + cudaGetErrorString(e));
   }
   if (rc) {

@@ -27,6 +27,7 @@ constexpr int MAXB = 32;       // instances per handle (the instance table trave
 constexpr int MAXSPAN = 192;   // block spans per launch
 constexpr int NTHR = 256;      // threads per block of every stage kernel
 constexpr int CT_BM = 64, CT_BK = 64;  // contingency tile: monitored branches x outages
+constexpr int HOT_BK = 4 * NTHR;        // outages per hot-row block of stage 2 (s2_hot)
 constexpr int DCF_BM = 32, DCF_TC = 8; // forward DC tile: 32 branches x 8 periods
 constexpr int PACK = 32;               // CSR entries per warp pack (rows never straddle packs)
 constexpr int PACKS_PER_BLOCK = NTHR / 32;
@@ -46,6 +47,9 @@ struct Inst {
   int bus0, br0, gen0, zone0, ctg0, gb0, tp0;
   int n_mt, n_kt;        // contingency tiles along monitored branches / outages
   int ctg_mg, n_mg;      // monitored-branch tiles per contingency block, and the number of such groups
+  int hot;               // stage 2 evaluates hot rows on their own (s2_hot): their column partial slots, one
+                         // per group of hot_mg tiles; 0: in the element screen
+  int hot_mg, hot_tb, hot_ntc; // 64-branch tiles and periods per hot-row block, and the number of period chunks
   int ctg_tb, ctg_ntc;   // periods per contingency block, and the number of period chunks
   int n_sb;              // stage-3 branch blocks per period (NTHR / InstTab::s3q branches each)
   int s4p;               // branch-end CSR packs per warp in stage 4 (1 or S4_PACKS)
@@ -57,6 +61,7 @@ struct Inst {
   long long pg0;         // PTDF restricted to generator buses: M x Gb, row m
   long long l0;          // line-outage block, M x Kp, row m
   long long pm0, pk0;    // contingency partials: [n_kt][T][M] and [n_mg][T][K]
+  long long ph0;         // column partials of the hot rows: [hot][T][Kp]
   long long pf0;         // flags of the row partials: [n_kt][T][n_mt], 1 where a 64-row tile has any
   long long lm0;         // bound-test row maxima of the line-outage block: [n_kt 4][n_mt 64]
   long long rm0;         // clearance minima per chunk of 8 periods (on-demand path): [ctg_ntc NCH][n_mt 64]
@@ -87,7 +92,7 @@ struct Inst {
 // the dense adjoint product with the device updates at each generator bus; R_SDCF / R_SDCA are their
 // counterparts around the sparse-factor solves (flows from the solved angles; right-hand side of
 // the adjoint solve), whose device updates are R_GEN / R_XF blocks of stage 5.
-enum Role : int { R_BRANCH = 0, R_ZONE, R_DCF, R_BUS, R_CTG, R_GBUS, R_GEN, R_SDCF, R_SDCA, R_XF, R_OBJ };
+enum Role : int { R_BRANCH = 0, R_ZONE, R_DCF, R_BUS, R_CTG, R_GBUS, R_GEN, R_SDCF, R_SDCA, R_XF, R_OBJ, R_HOT };
 
 constexpr int SP_RB = 64;   // dense tail product: rows per block
 constexpr int SP_BK = 32;   // dense tail product: columns per shared-memory chunk
@@ -125,7 +130,7 @@ struct Dev {
   // network (global ids)
   const int2 *br_end;                 // [sum M] (from, to) bus ids local to the instance
   const int *br_kidx;                 // [sum M] outage index of the branch within its instance, -1 if none
-  const Real *br_g, *br_b, *br_hch, *br_smax, *br_s2ctg;  // g_sr, b_sr, b_ch / 2, s_max, s_ctg^2
+  const Real *br_g, *br_b, *br_hch, *br_smax, *br_s2ctg, *br_sctg;  // g_sr, b_sr, b_ch / 2, s_max, s_ctg^2 and its square root
   const int *gen_bus, *gen_zone, *gen_gb;                 // local bus, local zone, local generator-bus index
   const Real *gen_a, *gen_b, *gen_cr, *gen_pmax;
   const Real *gen_sgn;                // +1 producer, -1 consumer (sign of p, q as supply)
@@ -206,6 +211,8 @@ struct Dev {
   Real *dP, *dQ;                      // [sum T n]
   Real *dZ;                           // [sum T Z]
   Real *pm, *pq, *pk;                 // contingency partials
+  unsigned char *hot;                 // [sum T M] 1: a hot row (its partials are s2_hot's)
+  Real *pkh, *pzh;                    // column (score) partials of the hot rows, [hot][T][Kp] per instance (pkh without the period's weight)
   unsigned char *pmf;                 // row-partial flags (pm, pq are written and read only where set)
   int score;                          // 1: record per-(period, outage) scores (contingency screening)
   Real *pz;                           // score partials [n_mg][T][K] per instance (at pk0)
@@ -243,6 +250,7 @@ struct Plan {
   long long n_x;
   int maxT;
   int maxTB;  // largest period chunk of a contingency block (sizes its shared memory)
+  int hot;        // stage 2 has hot-row blocks
   int ctg_bound;  // stage 2 runs its bound test (eager or on-demand path; the same for every instance)
   int ctg_lazy;   // stage 2 takes the on-demand path (k_ctg_margin runs before it)
   int n_gen_slots;  // objective reduction slots of the stage-5 device blocks
@@ -275,7 +283,7 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *x, bo
                         cudaStream_t s, cudaEvent_t *ev);
 
 template <typename Real, typename Dc>
-cudaError_t prepare_eval(int maxTB, bool score, bool lazy);
+cudaError_t prepare_eval(int maxTB, bool score, bool lazy, bool hot);
 
 // Row maxima of instance I's line-outage block for the stage-2 bound test (Dev::lmax at I.lm0), from
 // the block as stored (lodf, of type dtype); rerun whenever the block changes.

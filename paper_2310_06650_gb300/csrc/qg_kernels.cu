@@ -26,6 +26,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <map>
@@ -867,6 +868,11 @@ __device__ __forceinline__ float ctg_qs(Real q2, Real s2) {
   else return (float)(q2 - s2);
 }
 
+// Whether a monitored branch is over its post-contingency limit in the base case already, by the
+// screen's own values (NaN included): a hot row, where nearly every outage is an overload.  Stage 2
+// evaluates hot rows densely (s2_hot) and leaves them out of its element screen and bound test.
+__device__ __forceinline__ bool row_hot(float f, float qs) { return !(__fmaf_rn(f, f, qs) < 0.f); }
+
 // Bound test of one thread's 4 rows over a chunk: Lmax fc < r for each row, with Lmax the rows' largest
 // |L| over the thread's 16-outage group, fc that group's largest |f_k| over the chunk and r the rows'
 // smallest clearance (all finite, so no NaN can arise).
@@ -911,11 +917,48 @@ __global__ void __launch_bounds__(NTHR) k_ctg_margin(const __grid_constant__ Dev
           q2[j] = d.qm2[idx];
         }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) r = fminf(r, clear_margin(f[j], ctg_qs<Real>(q2[j], s2)));
+        for (int j = 0; j < 8; ++j) {
+          const float qs = ctg_qs<Real>(q2[j], s2);
+          r = fminf(r, I.hot && row_hot(f[j], qs) ? FLT_MAX : clear_margin(f[j], qs));  // hot rows are s2_hot's
+        }
       }
       d.ctg_rmin[I.rm0 + e] = r;
     }
   }
+}
+
+// An overloaded element (Eqs. sfr_pen-zctg): s = sqrt(a2), u = s - s_ctg, and through reciprocal square
+// roots val = sigma_s(u) and dd = w sigma'(u) / s, where dz/dF = dd F and dz/dqmax2 = dd / 2 (a few
+// units in the last place; on the FP64 path about half the instructions of square root, division and
+// square root, each a long sequence on GB300's FP64 pipe).  a2 > s_ctg^2 >= 0; infinities take the
+// plain forms, so that they propagate as they would there.
+__device__ __forceinline__ void ctg_element(double a2, double sctg, double eps, double w, double &val, double &dd) {
+  if (a2 < (double)INFINITY) {
+    const double ra = rsqrt(a2);
+    const double u = fmax(fma(a2, ra, -sctg), 0.0);
+    const double b2 = fma(u, u, eps * eps);
+    if (b2 > 0.0) {
+      const double rb = rsqrt(b2);
+      val = b2 * rb;
+      dd = w * (u * rb) * ra;
+    } else {
+      val = 0.0;
+      dd = 0.0;
+    }
+  } else {
+    const double sv = sqrt(a2);
+    double der;
+    soft_relu(sv - sctg, eps, val, der);
+    dd = w * der / sv;
+  }
+}
+__device__ __forceinline__ void ctg_element(float a2, float sctg, float eps, float w, float &val, float &dd) {
+  const float ra = rsqrtf(a2);
+  const float u = fmaxf(__fmaf_rn(a2, ra, -sctg), 0.f);
+  const float b2 = __fmaf_rn(u, u, eps * eps);
+  const float rb = rsqrtf(b2);
+  val = b2 * rb;  // sqrt(u^2 + eps^2)
+  dd = w * (u * rb) * ra;
 }
 
 // Contingency block (Sec. II-E, Eqs. rank_correct, sfr_pen-zctg) for outages [k0, k0 + 64), the
@@ -1145,6 +1188,10 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
             const long long idx = I.tm0 + (long long)(t0 + tt) * I.M + m;
             f = d.f32[idx];
             qs = ctg_qs<Real>(d.qm2[idx], d.br_s2ctg[I.br0 + m]);
+            if (I.hot && row_hot(f, qs)) {  // s2_hot's row: F^2 - inf is never a candidate
+              f = 0.f;
+              qs = -INFINITY;
+            }
             if (F64) f64 = d.fre[idx];
           }
           s_fm[tt * CT_BM + c] = f;
@@ -1173,7 +1220,12 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
             f = d.f32[idx];
             qs = ctg_qs<Real>(d.qm2[idx], s2);
             if (F64) f64 = d.fre[idx];
-            rmin = fminf(rmin, clear_margin(f, qs));
+            if (I.hot && row_hot(f, qs)) {
+              f = 0.f;
+              qs = -INFINITY;
+            } else {
+              rmin = fminf(rmin, clear_margin(f, qs));
+            }
           }
           s_fm[tt * CT_BM + sc] = f;
           s_qs[tt * CT_BM + sc] = qs;
@@ -1257,34 +1309,23 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
               for (int j = 0; j < 4; ++j) {
                 if (!(F64 ? y[i][j] >= 0.f : y[i][j] > 0.f)) continue;  // NaN (pad, outaged branch) fails too
                 const Real q2 = d.qm2[I.tm0 + (long long)(t0 + tl) * I.M + m0 + mm];
-                Real Fx, Lx, sv, dd;
+                Real Fx, Lx, dd;
+                Real val;
                 if (F64) {
                   Lx = (Real)d.lodf64[I.l0 + (long long)(m0 + mm) * I.Kp + kc + j];
                   Fx = s_f64m[tl * CT_BM + mm] + Lx * s_f64k[tl * CT_BK + cq * 4 + j];
-                  if (Fx * Fx + q2 - s_s2[mm] <= Real(0)) continue;
-                  sv = dsqrt(Fx * Fx + q2);
-                  Real val, der;
-                  soft_relu(sv - s_s2[CT_BM + mm], eps, val, der);
-                  obj += w * (val - eps);
-                  zc[j] += w * (val - eps);
-                  dd = w * der / sv;  // dz/dF = w sigma' F / s
+                  const Real a2 = Fx * Fx + q2;
+                  if (a2 - s_s2[mm] <= Real(0)) continue;
+                  ctg_element(a2, s_s2[CT_BM + mm], eps, w, val, dd);
                 } else {
-                  // mixed path: s = sqrt(F^2 + qmax2) and the soft-ReLU through reciprocal square
-                  // roots (a few units in the last place, below the FP32 error of F itself)
                   float l0, l1;
                   unpack2(Lp[i >> 1][j], l0, l1);
                   Lx = (i & 1) ? l1 : l0;
                   Fx = F[i][j];
-                  const float a2 = __fmaf_rn(F[i][j], F[i][j], (float)q2);
-                  const float ra = rsqrtf(a2);
-                  const float u = fmaxf(__fmaf_rn(a2, ra, -(float)s_s2[CT_BM + mm]), 0.f);
-                  const float b2 = __fmaf_rn(u, u, (float)(eps * eps));
-                  const float rb = rsqrtf(b2);
-                  const float val = b2 * rb;  // sqrt(u^2 + eps^2)
-                  obj += w * (val - eps);
-                  zc[j] += w * (val - eps);
-                  dd = w * (u * rb) * ra;  // w sigma'(s - s_ctg) / s
+                  ctg_element(Real(__fmaf_rn(F[i][j], F[i][j], (float)q2)), s_s2[CT_BM + mm], eps, w, val, dd);
                 }
+                obj += w * (val - eps);
+                zc[j] += w * (val - eps);
                 gm[i] += dd * Fx;
                 gk[j] += dd * Fx * Lx;
                 gq[i] += Real(0.5) * dd;     // dz/dqmax2 = w sigma' / (2 s)
@@ -1339,7 +1380,7 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
         for (int e = threadIdx.x; e < tn * CT_BM; e += NTHR) {
           const int tt = e / CT_BM, c = e % CT_BM, m = m0 + c;
           if (!s_hit[tt]) continue;
-          if (m < I.M) {
+          if (m < I.M && s_qs[(tc0 + tt) * CT_BM + c] != -INFINITY) {  // hot rows' partials are s2_hot's
             const long long q = I.pm0 + ((long long)kt * T + t0 + tc0 + tt) * I.M + m;
             d.pm[q] = s_gm[e];
             d.pq[q] = s_gq[e];
@@ -1386,6 +1427,264 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
   acc.v[0] = DcOps<Dc>::from_real(obj);
 }
 
+// Hot rows (row_hot) over every outage (plans with Inst::hot).  At an iterate about 1% of the branches
+// are over their limit before any outage, and they hold 92-99% of the overloaded elements; in the
+// element screen each would keep half a warp busy and its tile's staging, barriers and flushes with it.
+// Here a block takes hot_mg tiles of monitored branches x hot_tb periods x HOT_BK outages, finds the
+// hot rows by ballots (one bit per row of a tile and period), lists them in (tile, period, row) order,
+// HOT_RB at a time with their scalars in shared memory, and walks the list with four consecutive outages
+// per thread: no idle lanes, no branch per element, the next row's loads in flight while the current one
+// is evaluated.  A row's sums go to its partial slot of the chunk's first outage tile (which the screen
+// leaves to this path), the column sums stay with their thread (in registers while the period lasts,
+// else in pkh, one owner per entry; without the period's weight, which stage 3 applies).  On the mixed path
+// the block covers what a contingency block covers and sums the objective per row quad and column quad in
+// the screen's order, so that its FP32 rounding stays that of one running sum per thread of such a block.
+constexpr int HOT_MASKS = 32;     // (tile, period) pairs per list
+constexpr int HOT_RB = 32;        // rows staged at a time
+
+// One listed row: its scalars (Real) and where it is.
+template <typename Real>
+struct HotRow {
+  Real f, q2, s2, sctg;
+  int m, tt, kx, quad;
+};
+
+template <typename Real>
+constexpr size_t hot_smem_bytes() {
+  return sizeof(Real) * ((sizeof(Real) == 4 ? (CT_BM / 4) * NTHR : 0) + HOT_RB * (NTHR / 32) * 2) +
+         sizeof(HotRow<Real>) * HOT_RB + sizeof(unsigned long long) * HOT_MASKS + sizeof(int) * HOT_MASKS * CT_BM;
+}
+
+// Four consecutive values at p, aligned to the four.
+__device__ __forceinline__ void load4(const float *p, float (&v)[4]) {
+  const float4 q = *reinterpret_cast<const float4 *>(p);
+  v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+__device__ __forceinline__ void load4(const double *p, double (&v)[4]) {
+  const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ void store4(float *p, const float (&v)[4]) {
+  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(double *p, const double (&v)[4]) {
+  reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+  reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+}
+
+// One element of a hot row: whether it is overloaded, sigma_s(u) (val) and sigma'(u) / s (dd, without the
+// weight).  The values are used only where it is.  The FP64 form keeps to about 20 instructions of the
+// FP64 pipe, what bounds this path there: signs are tested on the integer pipe.
+__device__ __forceinline__ bool hot_element(double F, double q2, double s2, double sctg, double eps, float, double &val,
+                                            double &dd) {
+  const double a2 = fma(F, F, q2);
+  const long long over = __double_as_longlong(a2 - s2);  // > 0 and not NaN: overloaded (infinities included)
+  if (over >= 0x7ff0000000000000LL) {  // an infinity (or NaN, never overloaded): plain forms propagate it
+    ctg_element(a2, sctg, eps, 1.0, val, dd);
+    return over == 0x7ff0000000000000LL;
+  }
+  const double ra = rsqrt(a2);
+  double u = fma(a2, ra, -sctg);
+  u = __double_as_longlong(u) < 0 ? 0.0 : u;
+  const double b2 = fma(u, u, eps * eps);
+  const double rb = __double_as_longlong(b2) > 0 ? rsqrt(b2) : 0.0;
+  val = b2 * rb;
+  dd = u * rb * ra;
+  return over > 0;
+}
+__device__ __forceinline__ bool hot_element(float F, float q2, float, float sctg, float eps, float qs, float &val, float &dd) {
+  ctg_element(__fmaf_rn(F, F, q2), sctg, eps, 1.f, val, dd);
+  return __fmaf_rn(F, F, qs) > 0.f;  // the screen's classification
+}
+
+template <typename Real, typename Dc>
+__device__ void s2_hot(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> &acc, const HP<Real> hp) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr bool F64 = sizeof(Real) == 8;
+  constexpr int NW = NTHR / 32;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int n_hc = (I.K + HOT_BK - 1) / HOT_BK;
+  const int hc = sub % n_hc, tci = (sub / n_hc) % I.hot_ntc, mg = sub / (n_hc * I.hot_ntc);
+  const int T = I.T, t0 = tci * I.hot_tb, TB = min(I.hot_tb, T - t0);
+  const int mt0 = mg * I.hot_mg, np = (min(I.n_mt, mt0 + I.hot_mg) - mt0) * TB;
+  const int kc = hc * HOT_BK + threadIdx.x * 4;
+  const bool col = kc < I.K;
+  HotRow<Real> *s_row = reinterpret_cast<HotRow<Real> *>(smem_raw);                        // [HOT_RB]
+  unsigned long long *s_mask = reinterpret_cast<unsigned long long *>(s_row + HOT_RB);     // [HOT_MASKS]
+  Real *s_red = reinterpret_cast<Real *>(s_mask + HOT_MASKS);                              // [HOT_RB][2][NW]
+  Real *s_obj = s_red + HOT_RB * NW * 2 + threadIdx.x;                                     // [row quad][NTHR], mixed path
+  int *s_list = reinterpret_cast<int *>(s_red + HOT_RB * NW * 2 + (F64 ? 0 : (CT_BM / 4) * NTHR));  // [HOT_MASKS CT_BM]
+  __shared__ int s_n;
+  const bool score = d.score != 0;
+  const Real eps = hp.eps;
+  Real *pk = d.pkh + I.ph0 + ((long long)mg * T + t0) * I.Kp + kc;  // this thread's columns, rows of Kp periods on
+  Real *pz = score ? d.pzh + I.ph0 + ((long long)mg * T + t0) * I.Kp + kc : nullptr;
+  if (!F64)
+#pragma unroll
+    for (int r = 0; r < CT_BM / 4; ++r) s_obj[r * NTHR] = 0;
+  Real obj = 0;  // FP64 path
+  pdl_wait();
+  if (col) {
+    const Real z4[4] = {0, 0, 0, 0};
+    for (int tt = 0; tt < TB; ++tt) {
+      store4(pk + (long long)tt * I.Kp, z4);
+      if (score) store4(pz + (long long)tt * I.Kp, z4);
+    }
+  }
+  Real gk[4] = {0, 0, 0, 0};  // the column sums of period tcur; those of the other periods are in pkh
+  int tcur = -1;
+  Real wt = 0;
+  for (int p0 = 0; p0 < np; p0 += HOT_MASKS) {
+    const int pn = min(np - p0, HOT_MASKS);
+    // the hot rows of each (tile, period) of the batch, one bit per row
+#pragma unroll
+    for (int e = wid; e < HOT_MASKS; e += NW) {
+      if (e >= pn) break;
+      const int mt = mt0 + (p0 + e) / TB, tt = (p0 + e) % TB, ma = mt * CT_BM + lane, mb = ma + 32;
+      const long long tm = I.tm0 + (long long)(t0 + tt) * I.M;
+      const bool ha = ma < I.M && row_hot(d.f32[tm + ma], ctg_qs<Real>(d.qm2[tm + ma], d.br_s2ctg[I.br0 + ma]));
+      const bool hb = mb < I.M && row_hot(d.f32[tm + mb], ctg_qs<Real>(d.qm2[tm + mb], d.br_s2ctg[I.br0 + mb]));
+      const unsigned ba = __ballot_sync(0xffffffffu, ha), bb = __ballot_sync(0xffffffffu, hb);
+      if (lane == 0) s_mask[e] = (unsigned long long)bb << 32 | ba;
+      if (hc == 0) {
+        if (ma < I.M) d.hot[tm + ma] = ha ? 1 : 0;
+        if (mb < I.M) d.hot[tm + mb] = hb ? 1 : 0;
+      }
+    }
+    __syncthreads();
+    if (wid == 0) {  // their list: place in the batch << 6 | row of the tile
+      unsigned long long mask = lane < pn ? s_mask[lane] : 0ull;
+      int pre = __popcll(mask);
+      const int own = pre;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, pre, o);
+        if (lane >= o) pre += v;
+      }
+      if (lane == 31) s_n = pre;
+      for (int q = pre - own; mask; mask &= mask - 1) s_list[q++] = lane << 6 | (__ffsll((long long)mask) - 1);
+    }
+    __syncthreads();
+    const int n = s_n;
+    for (int i0 = 0; i0 < n; i0 += HOT_RB) {
+      const int rn = min(HOT_RB, n - i0);
+      if ((int)threadIdx.x < rn) {
+        const int v = s_list[i0 + threadIdx.x], p = p0 + (v >> 6), tt = p % TB, m = (mt0 + p / TB) * CT_BM + (v & 63);
+        const long long e = I.tm0 + (long long)(t0 + tt) * I.M + m;
+        HotRow<Real> r;
+        r.f = F64 ? d.fre[e] : (Real)d.f32[e];
+        r.q2 = d.qm2[e];
+        r.s2 = d.br_s2ctg[I.br0 + m];
+        r.sctg = d.br_sctg[I.br0 + m];
+        r.m = m;
+        r.tt = tt;
+        r.kx = d.br_kidx[I.br0 + m];
+        r.quad = (v & 63) >> 2;
+        s_row[threadIdx.x] = r;
+      }
+      __syncthreads();
+      Real Ln[4] = {0, 0, 0, 0}, fn[4] = {0, 0, 0, 0};
+      auto fetch = [&](int i) {  // the line-outage and flow values of row i
+        if (!col) return;
+        const int m = s_row[i].m, tt = s_row[i].tt;
+        const long long l = I.l0 + (long long)m * I.Kp + kc;  // rows are padded to 4 columns
+        if constexpr (F64) load4(d.lodf64 + l, Ln);
+        else lodf_load4(d.lodf, l, d.lodf_dtype, Ln);
+        const long long ek = I.tk0 + (long long)(t0 + tt) * I.K + kc;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (kc + j < I.K) fn[j] = F64 ? d.fk[ek + j] : (Real)d.fk32[ek + j];
+      };
+      fetch(0);
+      if (s_row[0].tt != tcur) {
+        if (col) {
+          if (tcur >= 0) store4(pk + (long long)tcur * I.Kp, gk);
+          load4(pk + (long long)s_row[0].tt * I.Kp, gk);
+        }
+        tcur = s_row[0].tt;
+        wt = d.dt[I.tp0 + t0 + tcur] * d.c_s * hp.beta;
+      }
+      for (int i = 0; i < rn; ++i) {
+        const HotRow<Real> h = s_row[i];
+        Real L[4], fk[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          L[j] = Ln[j];
+          fk[j] = fn[j];
+        }
+        const int inext = min(i + 1, rn - 1), tnext = s_row[inext].tt;
+        if (i + 1 < rn) fetch(i + 1);
+        Real gn[4] = {0, 0, 0, 0}, wn = wt;
+        if (tnext != tcur) {  // the next row is another period's (not the one whose sums are in registers)
+          if (col) load4(pk + (long long)tnext * I.Kp, gn);
+          wn = d.dt[I.tp0 + t0 + tnext] * d.c_s * hp.beta;
+        }
+        Real gm = 0, gq = 0;
+        if (col) {
+          Real gz[4];
+          if (score) load4(pz + (long long)h.tt * I.Kp, gz);
+          Real o = F64 ? obj : s_obj[h.quad * NTHR];
+          const float qs = ctg_qs<Real>(h.q2, h.s2);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const Real F = F64 ? h.f + L[j] * fk[j] : (Real)__fmaf_rn((float)L[j], (float)fk[j], (float)h.f);
+            Real val, dd;
+            // a pad, and the outaged branch itself, are not monitored
+            const bool over = hot_element(F, h.q2, h.s2, h.sctg, eps, qs, val, dd) && kc + j < I.K && kc + j != h.kx;
+            const Real z = over ? wt * (val - eps) : Real(0);
+            dd = over ? dd : Real(0);
+            const Real dF = over ? dd * F : Real(0);
+            o += z;
+            gm += dF;
+            gq += dd;
+            gk[j] += over ? dF * L[j] : Real(0);
+            if (score) gz[j] += z;
+          }
+          if (F64) obj = o;
+          else s_obj[h.quad * NTHR] = o;
+          if (score) store4(pz + (long long)h.tt * I.Kp, gz);
+        }
+        // the row's sums over the warp: lanes below 16 finish gm, the others gq
+        const bool up = lane & 16;
+        Real v = (up ? gq : gm) + __shfl_xor_sync(0xffffffffu, up ? gm : gq, 16);
+#pragma unroll
+        for (int q = 8; q > 0; q >>= 1) v += __shfl_xor_sync(0xffffffffu, v, q);
+        if ((lane & 15) == 0) s_red[(2 * i + (lane >> 4)) * NW + wid] = (up ? Real(0.5) * wt : wt) * v;
+        if (tnext != tcur) {
+          if (col) {
+            store4(pk + (long long)tcur * I.Kp, gk);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) gk[j] = gn[j];
+          }
+          tcur = tnext;
+          wt = wn;
+        }
+      }
+      __syncthreads();
+      if ((int)threadIdx.x < 2 * rn) {  // the rows' sums over the warps, in order
+        const Real *v = s_red + threadIdx.x * NW;
+        Real a = v[0];
+#pragma unroll
+        for (int q = 1; q < NW; ++q) a += v[q];
+        const HotRow<Real> &r = s_row[threadIdx.x >> 1];
+        const long long q = I.pm0 + ((long long)(hc * (HOT_BK / CT_BK)) * T + t0 + r.tt) * I.M + r.m;
+        if (threadIdx.x & 1) d.pq[q] = a;
+        else d.pm[q] = a;
+      }
+      __syncthreads();
+    }
+  }
+  if (col && tcur >= 0) store4(pk + (long long)tcur * I.Kp, gk);
+  if (F64) {
+    acc.v[0] = DcOps<Dc>::from_real(obj);
+  } else {
+    Dc sum = DcOps<Dc>::zero();
+#pragma unroll
+    for (int r = 0; r < CT_BM / 4; ++r) sum = DcOps<Dc>::add(sum, DcOps<Dc>::from_real(s_obj[r * NTHR]));
+    acc.v[0] = sum;
+  }
+}
+
 template <typename Real, typename Dc, int MODE>
 __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s2(const __grid_constant__ Dev<Real, Dc> d,
                                              const __grid_constant__ InstTab tab, const __grid_constant__ Spans S,
@@ -1397,6 +1696,9 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s2(const __
     acc.id[0] = T_ZP;
     acc.id[1] = T_ZQ;
     s2_bus(d, I, w.t, w.sub, x, acc, hparams(d));  // waits after its static loads
+  } else if (w.role == R_HOT) {
+    acc.id[0] = T_ZCTG;
+    s2_hot(d, I, w.sub, acc, hparams(d));
   } else {
     acc.id[0] = T_ZCTG;
     s2_ctg<Real, Dc, MODE>(d, I, w.sub, acc, hparams(d));
@@ -1516,35 +1818,76 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       phi = x[I.xtau0 + (long long)(I.T + t) * I.X + xi0];
     }
   }
-  Real gF = 0, gq2 = 0, gk = 0, zk = 0;
-  if (on) {
-    // row partials of the outage tiles whose 64-row tile had an overload (flagged by stage 2): few
-    // tiles are read unconditionally and selected (no dependent load), many are skipped
-    if (I.n_kt <= 16 * SPLIT) {
-#pragma unroll 4
-      for (int kt = q; kt < I.n_kt; kt += SPLIT) {
-        const long long pq = I.pm0 + ((long long)kt * I.T + t) * I.M + j;
-        const bool f = d.pmf[I.pf0 + ((long long)kt * I.T + t) * I.n_mt + (j >> 6)] != 0;
-        const Real a = d.pm[pq], b = d.pq[pq];
-        gF += f ? a : Real(0);
-        gq2 += f ? b : Real(0);
+  const Real wctg = d.dt[I.tp0 + t] * d.c_s * hparams(d).beta;  // the hot rows' column sums come without it
+  Real gF = 0, gq2 = 0, gk = 0, gh = 0, zk = 0;  // gh: the hot rows' share of gk
+  // row partials of the outage tiles whose 64-row tile had an overload (flagged by stage 2), or, for a hot
+  // row, of the first outage tile of each of s2_hot's chunks: few tiles are read unconditionally and
+  // selected (no dependent load); of many, the set ones are summed in order
+  const bool hot = on && I.hot && d.hot[e] != 0;
+  if (I.n_kt > 16 * SPLIT) {
+    for (int k0 = 0; k0 < I.n_kt; k0 += 32) {
+      unsigned set = 0;
+      if (SPLIT == 1) {  // the warp's branches share one 64-row tile: lane l loads the flag of outage tile k0 + l
+        const int kl = k0 + (threadIdx.x & 31), tile = min(j & ~31, I.M - 1) >> 6;
+        set = __ballot_sync(0xffffffffu, kl < I.n_kt && d.pmf[I.pf0 + ((long long)kl * I.T + t) * I.n_mt + tile] != 0);
+      } else if (on) {
+        for (int kt = k0; kt < min(I.n_kt, k0 + 32); ++kt)
+          if (kt % SPLIT == q && d.pmf[I.pf0 + ((long long)kt * I.T + t) * I.n_mt + (j >> 6)]) set |= 1u << (kt - k0);
       }
-    } else {
-      for (int kt = q; kt < I.n_kt; kt += SPLIT) {
-        if (!d.pmf[I.pf0 + ((long long)kt * I.T + t) * I.n_mt + (j >> 6)]) continue;
-        const long long pq = I.pm0 + ((long long)kt * I.T + t) * I.M + j;
+      if (hot) {
+        set = 0;
+        for (int kt = k0; kt < min(I.n_kt, k0 + 32); kt += HOT_BK / CT_BK)
+          if (kt % SPLIT == q) set |= 1u << (kt - k0);
+      }
+      for (set = on ? set : 0; set; set &= set - 1) {
+        const long long pq = I.pm0 + ((long long)(k0 + __ffs(set) - 1) * I.T + t) * I.M + j;
         gF += d.pm[pq];
         gq2 += d.pq[pq];
       }
     }
+  }
+  if (on) {
+    if (I.n_kt <= 16 * SPLIT) {
+#pragma unroll 4
+      for (int kt = q; kt < I.n_kt; kt += SPLIT) {
+        const long long pq = I.pm0 + ((long long)kt * I.T + t) * I.M + j;
+        const bool flag = d.pmf[I.pf0 + ((long long)kt * I.T + t) * I.n_mt + (j >> 6)] != 0;
+        const bool f = hot ? kt % (HOT_BK / CT_BK) == 0 : flag;
+        const Real a = d.pm[pq], b = d.pq[pq];
+        gF += f ? a : Real(0);
+        gq2 += f ? b : Real(0);
+      }
+    }
     if (kx >= 0) {
+      if (SPLIT > 1 || I.n_mg + I.hot <= 32) {
 #pragma unroll 8
-      for (int mg = q; mg < I.n_mg; mg += SPLIT) gk += d.pk[I.pk0 + ((long long)mg * I.T + t) * I.K + kx];
-      if (d.score)
+        for (int mg = q; mg < I.n_mg; mg += SPLIT) gk += d.pk[I.pk0 + ((long long)mg * I.T + t) * I.K + kx];
+#pragma unroll 8
+        for (int mg = q; mg < I.hot; mg += SPLIT) gh += d.pkh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + kx];
+      }
+      if (d.score) {
         for (int mg = q; mg < I.n_mg; mg += SPLIT) zk += d.pz[I.pk0 + ((long long)mg * I.T + t) * I.K + kx];
+        for (int mg = q; mg < I.hot; mg += SPLIT) zk += d.pzh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + kx];
+      }
     }
   }
+  if (SPLIT == 1 && I.n_mg + I.hot > 32) {
+    // many column partials (large plans, where few branches are outages): the whole warp sums those of
+    // each of its outage branches, a lane every 32nd, instead of one lane walking them all
+    const int lane = threadIdx.x & 31;
+    for (unsigned todo = __ballot_sync(0xffffffffu, on && kx >= 0); todo; todo &= todo - 1) {
+      const int src = __ffs(todo) - 1, k = __shfl_sync(0xffffffffu, kx, src);
+      Real s = 0;
+#pragma unroll 2
+      for (int mg = lane; mg < I.n_mg; mg += 32) s += d.pk[I.pk0 + ((long long)mg * I.T + t) * I.K + k];
+#pragma unroll 4
+      for (int mg = lane; mg < I.hot; mg += 32) s += wctg * d.pkh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + k];
 #pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == src) gk = s;
+    }
+  }
+  gk += gh * wctg;
 #pragma unroll
   for (int o = 1; o < SPLIT; o <<= 1) {
     gF += __shfl_xor_sync(0xffffffffu, gF, o);
@@ -2501,15 +2844,16 @@ __global__ void __launch_bounds__(NTHR) k_sp_back(const __grid_constant__ Dev<Re
 // ---------------------------------------------------------------------------------------------
 
 template <typename Real>
-size_t ctg_smem_bytes(int TB, bool score, bool lazy) {
+size_t ctg_smem_bytes(int TB, bool score, bool lazy, bool hot) {
   constexpr bool F64 = sizeof(Real) == 8;
   constexpr int TCH = ctg_tch<Real>();
   const size_t nch = (TB + TCH - 1) / TCH;
-  return sizeof(float) * ((size_t)TB * (2 * CT_BM + 2 * CT_BK) + nch * (CT_BM + 4) +
+  const size_t ctg = sizeof(float) * ((size_t)TB * (2 * CT_BM + 2 * CT_BK) + nch * (CT_BM + 4) +
                           (lazy ? (size_t)CT_TBATCH * (4 + nch) * CT_BM : 0)) +
          sizeof(Real) * ((size_t)TB * CT_BK + 2 * CT_BM + (size_t)TCH * (2 * CT_BM + 8 * CT_BK) +
                          (F64 ? (size_t)TB * (CT_BM + CT_BK) : 0) +
                          (score ? (size_t)TCH * 8 * CT_BK + (size_t)TB * CT_BK : 0));
+  return hot ? std::max(ctg, hot_smem_bytes<Real>()) : ctg;  // the hot-row blocks run in the same launch
 }
 
 // Record a timing event on s; inside stream capture it becomes an external event node.
@@ -2592,7 +2936,7 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
   nvtxRangePushA("qg stage 2 (contingencies)");
   if (P.s2.n_blocks > 0) {  // no contingencies: nothing for stage 2
     if (P.ctg_lazy) go(k_ctg_margin<Real, Dc>, 152 * 4, 0, d, P.tab);
-    const size_t sm2 = ctg_smem_bytes<Real>(P.maxTB, d.score != 0, P.ctg_lazy != 0);
+    const size_t sm2 = ctg_smem_bytes<Real>(P.maxTB, d.score != 0, P.ctg_lazy != 0, P.hot != 0);
     if (P.ctg_lazy) go(k_s2<Real, Dc, 2>, P.s2.n_blocks, sm2, d, P.tab, P.s2, (const Real *)x, o2);
     else if (P.ctg_bound) go(k_s2<Real, Dc, 1>, P.s2.n_blocks, sm2, d, P.tab, P.s2, (const Real *)x, o2);
     else go(k_s2<Real, Dc, 0>, P.s2.n_blocks, sm2, d, P.tab, P.s2, (const Real *)x, o2);
@@ -2638,10 +2982,10 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
 // The contingency kernel's dynamic shared-memory limit is a process-wide function attribute: it is
 // only ever raised, so that creating a handle with smaller blocks never breaks an existing one.
 template <typename Real, typename Dc>
-cudaError_t prepare_eval(int maxTB, bool score, bool lazy) {
+cudaError_t prepare_eval(int maxTB, bool score, bool lazy, bool hot) {
   static std::mutex mu;
   static size_t cur = 0;  // the same limit for every instantiation
-  const size_t sm = ctg_smem_bytes<Real>(maxTB, score, lazy);
+  const size_t sm = ctg_smem_bytes<Real>(maxTB, score, lazy, hot);
   if (sm > 227 * 1024) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(mu);
   if (sm <= cur) return cudaSuccess;
@@ -2807,10 +3151,10 @@ template cudaError_t launch_eval<double, double>(const Dev<double, double> &, co
                                                  bool, cudaStream_t, cudaEvent_t *);
 template cudaError_t launch_eval<float, df32>(const Dev<float, df32> &, const Plan &, const void *, bool, bool,
                                               cudaStream_t, cudaEvent_t *);
-template cudaError_t prepare_eval<double, double>(int, bool, bool);
+template cudaError_t prepare_eval<double, double>(int, bool, bool, bool);
 template cudaError_t launch_finish<double, double>(const Dev<double, double> &, const Plan &, int, cudaStream_t);
 template cudaError_t launch_finish<float, df32>(const Dev<float, df32> &, const Plan &, int, cudaStream_t);
-template cudaError_t prepare_eval<float, df32>(int, bool, bool);
+template cudaError_t prepare_eval<float, df32>(int, bool, bool, bool);
 template cudaError_t launch_adam<double>(double *, double *, double *, const double *, const double *, const double *,
                                          long long, long long *, unsigned int *, double, double, double, double, int,
                                          cudaStream_t);
