@@ -150,8 +150,9 @@ constexpr size_t umma_smem_bytes() {
 //   sum over the K blocks [s kbps, (s + 1) kbps) of A[m][k] B[n][k],
 // A (M x K) and B (N x K) BF16 behind the tensor maps tA (box 64 x 128) and tB (box 64 x BN); rows
 // and K beyond the tensors read as zeros.  Grid (ceil(M/128), ceil(N/BN), splits), 128 threads.
-// Launched as a programmatic dependent of the previous kernel: with a_static (A is not written by
-// the two kernels before it: the weights) the first stages' A tiles are requested before the wait.
+// Launched as a programmatic dependent of the previous kernel: with a_static (A, the weights, is not
+// written by the previous kernel, every block of which has waited for the kernels before it) the first
+// stages' A tiles are requested before the wait.
 // A wait that runs out sets *err, drains what this block started and returns.
 template <int BN, int STAGES>
 __global__ void __launch_bounds__(UTHREADS, 1)
@@ -286,104 +287,187 @@ __global__ void __launch_bounds__(UTHREADS, 1)
   }
 }
 
-// Transposed BF16 copy: dst[c][r] (row stride ldd) = src[r][c] (FP32, rows x cols, row stride lds),
-// through a 32 x 33 shared tile so that both sides are coalesced.  Grid (ceil(cols/32), ceil(rows/32)),
-// block (32, 8).
-__global__ void k_transpose_bf16(const float *__restrict__ src, long long lds, __nv_bfloat16 *__restrict__ dst,
-                                 long long ldd, int rows, int cols) {
-  pdl_wait();
-  __shared__ float t[32][33];
-  const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int r = r0 + i, c = c0 + threadIdx.x;
-    t[i][threadIdx.x] = (r < rows && c < cols) ? src[(long long)r * lds + c] : 0.f;
+// One 64 x 64 tile of a BF16 operand copy from the values v of this thread (rows wid + 8 i, columns
+// 2 lane and 2 lane + 1 of the tile): row-major with row stride ldd (dst) and, when dstT is given,
+// transposed with row stride ldt through shared memory, so that both are written in whole 128-byte lines.
+// Row strides are multiples of 8 (pad8) and the tile starts on even rows and columns, so pairs are aligned.
+// Called by all 256 threads of the block.
+__device__ __forceinline__ void store_tile_bf16(const float2 (&v)[8], __nv_bfloat16 *__restrict__ dst, long long ldd,
+                                                __nv_bfloat16 *__restrict__ dstT, long long ldt, int r0, int c0, int rows,
+                                                int cols) {
+  __shared__ __nv_bfloat16 t[64][66];  // [column][row]; 33 words per column: no bank conflict either way
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = wid + 8 * i, c = 2 * lane;
+    const __nv_bfloat162 h = __floats2bfloat162_rn(v[i].x, v[i].y);
+    if (dst && r0 + r < rows) {
+      __nv_bfloat16 *q = dst + (long long)(r0 + r) * ldd + c0 + c;
+      if (c0 + c + 1 < cols) *reinterpret_cast<__nv_bfloat162 *>(q) = h;
+      else if (c0 + c < cols) *q = h.x;
+    }
+    if (dstT) {
+      t[c][r] = h.x;
+      t[c + 1][r] = h.y;
+    }
   }
+  if (!dstT) return;
   __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += 8) {
-    const int c = c0 + i, r = r0 + threadIdx.x;
-    if (c < cols && r < rows) dst[(long long)c * ldd + r] = __float2bfloat16_rn(t[threadIdx.x][i]);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int c = wid + 8 * i, r = 2 * lane;
+    if (c0 + c >= cols) continue;
+    __nv_bfloat16 *q = dstT + (long long)(c0 + c) * ldt + r0 + r;
+    if (r0 + r + 1 < rows) *reinterpret_cast<__nv_bfloat162 *>(q) = *reinterpret_cast<const __nv_bfloat162 *>(&t[c][r]);
+    else if (r0 + r < rows) *q = t[c][r];
   }
 }
 
-// BF16 copy with a padded row stride: dst[r][c] (stride ldd) = src[r][c] (FP32, stride lds).
-// Grid (column chunks of 256, rows; the rows strided by gridDim.y): no index division per element.
-__global__ void k_rows_bf16(const float *__restrict__ src, long long lds, __nv_bfloat16 *__restrict__ dst, long long ldd,
-                            int rows, int cols) {
-  pdl_wait();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
-  for (int r = blockIdx.y; r < rows; r += gridDim.y) dst[(long long)r * ldd + c] = __float2bfloat16_rn(src[(long long)r * lds + c]);
-}
-
-// Epilogue of the forward layers: Z = sum of split-K partials + bias (M x N); optionally ReLU;
-// writes Z (FP32) and the activation in BF16 for the next GEMMs: row-major with row stride ldh
-// (Hb) and transposed with row stride ldt (HbT, batch-contiguous).
-__global__ void k_fwd_epi(const float *__restrict__ P, int splits, const float *__restrict__ bias, float *__restrict__ Z,
-                          __nv_bfloat16 *__restrict__ Hb, long long ldh, __nv_bfloat16 *__restrict__ HbT, long long ldt,
-                          int M, int N, int relu) {
-  pdl_wait();
-  const long long total = (long long)M * N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    float z = 0.f;
-    for (int s = 0; s < splits; ++s) z += P[s * total + i];
-    const long long r = i / N, c = i - r * N;
-    z += bias[c];
-    Z[i] = z;
-    const __nv_bfloat16 h = __float2bfloat16_rn(relu ? fmaxf(z, 0.f) : z);
-    if (Hb) Hb[r * ldh + c] = h;
-    if (HbT) HbT[c * ldt + r] = h;
-  }
-}
-
-// Backward epilogue: D = sum of split-K partials (rows x cols), masked by relu'(Zmask) when given;
-// FP32 (D, dense), BF16 row-major with row stride ldd (Db) and BF16 transposed with row stride
-// ldt (DbT).
-__global__ void k_bwd_epi(const float *__restrict__ P, int splits, const float *__restrict__ Zmask, float *__restrict__ D,
-                          __nv_bfloat16 *__restrict__ Db, long long ldd, __nv_bfloat16 *__restrict__ DbT, long long ldt,
-                          int rows, int cols) {
-  pdl_wait();
-  const long long total = (long long)rows * cols;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    float v = 0.f;
-    for (int s = 0; s < splits; ++s) v += P[s * total + i];
-    if (Zmask && !(Zmask[i] > 0.f)) v = 0.f;
-    if (D) D[i] = v;
-    if (Db || DbT) {
-      const long long r = i / cols, c = i - r * cols;
-      const __nv_bfloat16 h = __float2bfloat16_rn(v);
-      if (Db) Db[r * ldd + c] = h;
-      if (DbT) DbT[c * ldt + r] = h;
+// The 64 x 64 tile at (r0, c0) of an FP32 matrix (rows x cols, row stride cols), zeros outside: this
+// thread's 8 pairs, all in flight together; 8-byte loads where every row starts on an even element.
+__device__ __forceinline__ void load_tile(const float *__restrict__ src, bool even, int r0, int c0, int rows, int cols,
+                                          float2 (&v)[8]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, c = c0 + 2 * lane;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = r0 + wid + 8 * i;
+    v[i] = make_float2(0.f, 0.f);
+    if (r >= rows) continue;
+    const float *q = src + (long long)r * cols + c;
+    if (even && c + 1 < cols) v[i] = *reinterpret_cast<const float2 *>(q);
+    else {
+      if (c < cols) v[i].x = q[0];
+      if (c + 1 < cols) v[i].y = q[1];
     }
   }
 }
 
-// dY = 2 (Y - target) / (B * N) (BF16 for the backward GEMMs) and per-block partial sums of the
-// squared error (FP64, fixed order).
-__global__ void __launch_bounds__(256) k_loss(const float *__restrict__ Y, const float *__restrict__ Tg,
-                                              __nv_bfloat16 *__restrict__ dYb, long long ldo,
-                                              __nv_bfloat16 *__restrict__ dYbT, long long ldt, float *__restrict__ dY,
-                                              double *part, int rows, int cols) {
+__device__ __forceinline__ bool even_rows(const float *p, int cols) {
+  return (cols & 1) == 0 && (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+}
+
+// BF16 operand copies of an FP32 matrix, row-major (stride ldd) and optionally transposed (stride ldt).
+// Grid (ceil(cols/64), ceil(rows/64)), 256 threads.
+__global__ void __launch_bounds__(256) k_tile_bf16(const float *__restrict__ src, __nv_bfloat16 *__restrict__ dst,
+                                                   long long ldd, __nv_bfloat16 *__restrict__ dstT, long long ldt,
+                                                   int rows, int cols) {
   pdl_wait();
+  float2 v[8];
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  load_tile(src, even_rows(src, cols), r0, c0, rows, cols, v);
+  store_tile_bf16(v, dst, ldd, dstT, ldt, r0, c0, rows, cols);
+}
+
+// Epilogue tile: MAX_B batch rows x TC columns of a layer's output per block of 256 threads; thread
+// (column tid % TC, rows tid / TC + (256 / TC) i) sums its elements' split-K partials in split order,
+// with all its rows' loads of a split in flight together.
+constexpr int MAX_B = 64;
+enum { EPI_HIDDEN, EPI_OUT, EPI_LOSS, EPI_BACK };
+
+struct EpiArgs {
+  const float *P;         // partials [splits][B][N]
+  int splits, B, N;
+  const float *bias;      // forward: added after the partials
+  float *Z;               // EPI_HIDDEN: pre-activation; EPI_OUT: the network's output
+  const float *target;    // EPI_LOSS
+  double *lpart;          // EPI_LOSS: the block's sum of squared errors
+  const float *zmask;     // EPI_BACK: elements where it is not positive are zeroed (relu')
+  float *bgrad;           // EPI_LOSS, EPI_BACK: bias gradient, the column's sum in row order
+  __nv_bfloat16 *Hb;      // BF16 operand for the next GEMMs, row-major with row stride ldh (may be NULL) ...
+  long long ldh;
+  __nv_bfloat16 *HbT;     // ... and transposed with row stride ldt
+  long long ldt;
+};
+
+// What bounds it: the partials' read from L2 (a few microseconds at 16 to 36 splits) and the launch.  One
+// kernel per layer: the loss's residual and gradient come with the last layer's epilogue (the output
+// is not written and read again: at the rt617 network 42 us in three kernels before), bias gradients with
+// the tile that holds the whole batch.
+template <int MODE, int TC>
+__global__ void __launch_bounds__(256) k_epi(const __grid_constant__ EpiArgs a) {
+  constexpr int RS = 256 / TC, NR = MAX_B / RS;  // row stride, rows per thread
+  __shared__ float s_v[MAX_B][TC + 1];
   __shared__ double red[8];
-  double acc = 0.0;
-  const long long total = (long long)rows * cols;
-  const float sc = 2.0f / (float)total;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const float r = Y[i] - Tg[i];
-    acc += (double)r * (double)r;
-    dY[i] = sc * r;
-    const long long b = i / cols, o = i - b * cols;
-    const __nv_bfloat16 h = __float2bfloat16_rn(sc * r);
-    dYb[b * ldo + o] = h;
-    dYbT[o * ldt + b] = h;
+  pdl_wait();
+  const int c = threadIdx.x % TC, r0 = threadIdx.x / TC, n = blockIdx.x * TC + c;
+  const bool on = n < a.N;
+  const int total = a.B * a.N;  // below 2^31: the host allocates 64 times it
+  // elements outside the layer read element 0: every load is unconditional, 16 partials in flight
+  constexpr int UN = 16 / NR;
+  int at[NR];
+  float v[NR], x[NR];
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int r = r0 + i * RS;
+    at[i] = on && r < a.B ? r * a.N + n : 0;
+    v[i] = 0.f;
+    x[i] = 0.f;
+    if (MODE == EPI_LOSS) x[i] = __ldg(a.target + at[i]);
+    if (MODE == EPI_BACK) x[i] = __ldg(a.zmask + at[i]);
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  const float bias = MODE != EPI_BACK ? __ldg(a.bias + (on ? n : 0)) : 0.f;
+  int sp = 0;
+  for (; sp + UN <= a.splits; sp += UN) {
+    float t[UN][NR];
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+#pragma unroll
+      for (int i = 0; i < NR; ++i) t[u][i] = __ldg(a.P + (long long)(sp + u) * total + at[i]);
+#pragma unroll
+    for (int u = 0; u < UN; ++u)
+#pragma unroll
+      for (int i = 0; i < NR; ++i) v[i] += t[u][i];
+  }
+  for (; sp < a.splits; ++sp)
+#pragma unroll
+    for (int i = 0; i < NR; ++i) v[i] += __ldg(a.P + (long long)sp * total + at[i]);
+  const float sc = 2.0f / (float)total;
+  double acc = 0.0;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int r = r0 + i * RS;
+    const bool live = on && r < a.B;
+    const int e = at[i];
+    if (MODE == EPI_BACK) {
+      if (!(x[i] > 0.f)) v[i] = 0.f;
+    } else {
+      v[i] += bias;
+      if (MODE == EPI_LOSS) {
+        const float d = live ? v[i] - x[i] : 0.f;
+        acc += (double)d * (double)d;
+        v[i] = sc * d;
+      } else {
+        if (live) a.Z[e] = v[i];
+        if (MODE == EPI_HIDDEN) v[i] = fmaxf(v[i], 0.f);
+      }
+    }
+    if (MODE != EPI_OUT) s_v[r][c] = live ? v[i] : 0.f;
+  }
+  if (MODE == EPI_OUT) return;
+  if (MODE == EPI_LOSS) {
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[w];
-    part[blockIdx.x] = s;
+  if (MODE == EPI_LOSS && threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w];
+    a.lpart[blockIdx.x] = t;
+  }
+  if ((MODE == EPI_LOSS || MODE == EPI_BACK) && threadIdx.x < TC && blockIdx.x * TC + threadIdx.x < a.N) {
+    float t = 0.f;
+    for (int r = 0; r < a.B; ++r) t += s_v[r][threadIdx.x];
+    a.bgrad[blockIdx.x * TC + threadIdx.x] = t;
+  }
+  if (a.Hb)
+    for (int e = threadIdx.x; e < a.B * TC; e += 256) {
+      const int r = e / TC, cc = e % TC;
+      if (blockIdx.x * TC + cc < a.N) a.Hb[r * a.ldh + blockIdx.x * TC + cc] = __float2bfloat16_rn(s_v[r][cc]);
+    }
+  for (int e = threadIdx.x; e < TC * MAX_B; e += 256) {  // consecutive threads: consecutive rows of one column
+    const int cc = e / MAX_B, r = e % MAX_B;
+    if (r < a.B && blockIdx.x * TC + cc < a.N)
+      a.HbT[(long long)(blockIdx.x * TC + cc) * a.ldt + r] = __float2bfloat16_rn(s_v[r][cc]);
   }
 }
 
@@ -404,28 +488,88 @@ __global__ void __launch_bounds__(256) k_loss_final(const double *part, int n, l
   }
 }
 
-// Bias gradient: column sums of D (B x N) in row order.
-__global__ void k_colsum(const float *__restrict__ D, int B, int N, float *__restrict__ out) {
-  pdl_wait();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= N) return;
-  float s = 0.f;
-  for (int r = 0; r < B; ++r) s += D[(long long)r * N + c];
-  out[c] = s;
+// Adam on the FP32 master parameters and the BF16 operand copies of the updated weights, in one pass:
+// blocks [0, n_tiles) take 64 x 64 tiles of the three weight matrices (gradient, weight and both
+// moments read, weight and moments written, with the row-major and the transposed BF16 copies from the same
+// registers), the rest the biases.  Bound by HBM: 32 bytes per weight.  At the rt617 network (40 M
+// weights) Adam and the five copy kernels took 220 + 187 us.
+struct AdamMat {
+  long long off;                        // the matrix in the parameter layout
+  int rows, cols, tile0, tiles_c;       // its first tile and tiles per row of tiles
+  __nv_bfloat16 *b;                     // BF16 copy, row stride ldb
+  long long ldb;
+  __nv_bfloat16 *t;                     // transposed copy (may be NULL), row stride ldt
+  long long ldt;
+};
+struct AdamArgs {
+  AdamMat m[3];
+  int n_tiles;
+  long long bias_off[3];
+  int bias_n[3];
+  float lr, b1, b2, c1, c2, eps;
+};
+
+// (The multiply-adds are spelled out, so that the rounding of a training run does not hang on the compiler.)
+__device__ __forceinline__ void adam1(const AdamArgs &a, float &w, float g, float &m, float &v) {
+  m = __fmaf_rn(1.f - a.b1, g, __fmul_rn(a.b1, m));
+  v = __fmaf_rn(__fmul_rn(1.f - a.b2, g), g, __fmul_rn(a.b2, v));
+  w -= a.lr * (m * a.c1) / (sqrtf(v * a.c2) + a.eps);
 }
 
-// Adam on the FP32 master parameters; the BF16 weight copies follow.
-__global__ void k_mlp_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v,
-                           long long n, float lr, float b1, float b2, float c1, float c2, float eps) {
+__global__ void __launch_bounds__(256, 2) k_mlp_adam(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
+                                                  float *__restrict__ v, const __grid_constant__ AdamArgs a) {
   pdl_wait();
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+  if ((int)blockIdx.x >= a.n_tiles) {  // biases
+    long long i = (long long)(blockIdx.x - a.n_tiles) * 256 + threadIdx.x;
+    for (int q = 0; q < 3; ++q) {
+      if (i < a.bias_n[q]) {
+        const long long e = a.bias_off[q] + i;
+        float wi = w[e], mi = m[e], vi = v[e];
+        adam1(a, wi, g[e], mi, vi);
+        w[e] = wi;
+        m[e] = mi;
+        v[e] = vi;
+        return;
+      }
+      i -= a.bias_n[q];
+    }
+    return;
   }
+  const int q = (int)blockIdx.x >= a.m[2].tile0 ? 2 : (int)blockIdx.x >= a.m[1].tile0 ? 1 : 0;
+  const AdamMat &M = a.m[q];
+  const int tile = blockIdx.x - M.tile0, r0 = tile / M.tiles_c * 64, c0 = tile % M.tiles_c * 64;
+  const bool even = even_rows(w + M.off, M.cols);  // the four arrays are 256-byte aligned: the same for all
+  float2 wv[8], gv[8], mv[8], vv[8];
+  load_tile(g + M.off, even, r0, c0, M.rows, M.cols, gv);
+  load_tile(m + M.off, even, r0, c0, M.rows, M.cols, mv);
+  load_tile(v + M.off, even, r0, c0, M.rows, M.cols, vv);
+  load_tile(w + M.off, even, r0, c0, M.rows, M.cols, wv);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, c = c0 + 2 * lane;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    adam1(a, wv[i].x, gv[i].x, mv[i].x, vv[i].x);
+    adam1(a, wv[i].y, gv[i].y, mv[i].y, vv[i].y);
+    const int r = r0 + wid + 8 * i;
+    if (r >= M.rows) continue;
+    const long long e = M.off + (long long)r * M.cols + c;
+    if (even && c + 1 < M.cols) {
+      *reinterpret_cast<float2 *>(w + e) = wv[i];
+      *reinterpret_cast<float2 *>(m + e) = mv[i];
+      *reinterpret_cast<float2 *>(v + e) = vv[i];
+    } else {
+      if (c < M.cols) {
+        w[e] = wv[i].x;
+        m[e] = mv[i].x;
+        v[e] = vv[i].x;
+      }
+      if (c + 1 < M.cols) {
+        w[e + 1] = wv[i].y;
+        m[e + 1] = mv[i].y;
+        v[e + 1] = vv[i].y;
+      }
+    }
+  }
+  store_tile_bf16(wv, M.b, M.ldb, M.t, M.ldt, r0, c0, M.rows, M.cols);
 }
 
 // Deterministic counter-based normal draws (Box-Muller on a splitmix64 stream) for the initial weights.
@@ -482,7 +626,7 @@ struct qg_mlp {
   __nv_bfloat16 *w1b = nullptr, *w2b = nullptr, *w3b = nullptr, *w2t = nullptr, *w3t = nullptr;
   __nv_bfloat16 *xb = nullptr, *xt = nullptr, *h1b = nullptr, *h1t = nullptr, *h2b = nullptr, *h2t = nullptr;
   __nv_bfloat16 *dyb = nullptr, *dyt = nullptr, *dz2b = nullptr, *dz2t = nullptr, *dz1t = nullptr;
-  float *z1 = nullptr, *z2 = nullptr, *y = nullptr, *dy = nullptr, *dz2 = nullptr, *dz1 = nullptr, *part = nullptr;
+  float *z1 = nullptr, *z2 = nullptr, *part = nullptr;
   double *lpart = nullptr;
   int *d_err = nullptr;  // set by a GEMM block whose pipeline wait ran out
   long long part_elems = 0;
@@ -553,7 +697,7 @@ cudaError_t umma_prepare() {
 // into mm->part: [splits][M][N], or [splits][N][M] with trans; with dst, C itself (one split) into dst.  Returns the number of splits, or 0
 // after recording an error.  Narrow products (N <= 64: the batch) take 64-column tiles and a
 // 4-stage ring; wide ones (the weight gradients, K = the batch) 256-column tiles and 2 stages.
-// a_static: A is a weight copy (not written by the kernels just before), requested before the wait.
+// a_static: A is a weight copy (not written by the kernel just before), requested before the wait.
 int gemm(qg_mlp *mm, const __nv_bfloat16 *A, long long lda, int M, const __nv_bfloat16 *B, long long ldb, int N, int K,
          bool trans, bool a_static, float *dst = nullptr) {
   const bool narrow = N <= 64;
@@ -590,46 +734,46 @@ int gemm(qg_mlp *mm, const __nv_bfloat16 *A, long long lda, int M, const __nv_bf
   return splits;
 }
 
+dim3 tiles64(long long rows, long long cols) { return dim3((unsigned)((cols + 63) / 64), (unsigned)((rows + 63) / 64)); }
+
 // x (batch x I, FP32) into the BF16 operand xb [B][ld_i] and, for training (the first layer's weight
 // gradient), xt [I][ld_b]
 void load_x(qg_mlp *m, const float *x, int B, bool transposed) {
-  pdl_launch(k_rows_bf16, dim3((m->n_in + 255) / 256, std::min(B, 65535)), dim3(256), 0, m->stream, x, m->n_in, m->xb,
-             m->ld_i, B, m->n_in);
-  if (transposed)
-    pdl_launch(k_transpose_bf16, dim3((m->n_in + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, m->stream, x, m->n_in, m->xt,
-               m->ld_b, B, m->n_in);
+  pdl_launch(k_tile_bf16, tiles64(B, m->n_in), dim3(256), 0, m->stream, x, m->xb, m->ld_i,
+             transposed ? m->xt : (__nv_bfloat16 *)nullptr, m->ld_b, B, m->n_in);
 }
 
-// Forward pass: the layers as C^T = W act^T (weights as the 128-row operand, the batch as N).
+// Columns per epilogue block: narrow tiles where the layer is narrow, so that its blocks fill the SMs.
+constexpr int EPI_TC_H = 8, EPI_TC_O = 32;
+
+template <int MODE, int TC>
+void epi(qg_mlp *m, const EpiArgs &a) {
+  pdl_launch(k_epi<MODE, TC>, dim3((a.N + TC - 1) / TC), dim3(256), 0, m->stream, a);
+}
+
+// The two hidden layers and the last layer's GEMM, as C^T = W act^T (weights as the 128-row operand, the
+// batch as N); returns the last GEMM's splits, or 0 after an error.
 int forward(qg_mlp *m, int B) {
   const int H = m->n_h, I = m->n_in, O = m->n_out;
   int s = gemm(m, m->w1b, m->ld_i, H, m->xb, m->ld_i, B, I, true, true);
-  if (!s) return QG_ERR_CUDA;
-  pdl_launch(k_fwd_epi, dim3(grid_for((long long)B * H)), dim3(256), 0, m->stream, m->part, s, m->w + m->o_b1, m->z1,
-             m->h1b, m->ld_h, m->h1t, m->ld_b, B, H, 1);
-  if (!(s = gemm(m, m->w2b, m->ld_h, H, m->h1b, m->ld_h, B, H, true, true))) return QG_ERR_CUDA;
-  pdl_launch(k_fwd_epi, dim3(grid_for((long long)B * H)), dim3(256), 0, m->stream, m->part, s, m->w + m->o_b2, m->z2,
-             m->h2b, m->ld_h, m->h2t, m->ld_b, B, H, 1);
-  if (!(s = gemm(m, m->w3b, m->ld_h, O, m->h2b, m->ld_h, B, H, true, true))) return QG_ERR_CUDA;
-  pdl_launch(k_fwd_epi, dim3(grid_for((long long)B * O)), dim3(256), 0, m->stream, m->part, s, m->w + m->o_b3, m->y,
-             nullptr, 0, nullptr, 0, B, O, 0);
-  return QG_OK;
+  if (!s) return 0;
+  EpiArgs a{};
+  a.P = m->part; a.B = B; a.N = H;
+  a.splits = s; a.bias = m->w + m->o_b1; a.Z = m->z1; a.Hb = m->h1b; a.ldh = m->ld_h; a.HbT = m->h1t; a.ldt = m->ld_b;
+  epi<EPI_HIDDEN, EPI_TC_H>(m, a);
+  if (!(s = gemm(m, m->w2b, m->ld_h, H, m->h1b, m->ld_h, B, H, true, true))) return 0;
+  a.splits = s; a.bias = m->w + m->o_b2; a.Z = m->z2; a.Hb = m->h2b; a.HbT = m->h2t;
+  epi<EPI_HIDDEN, EPI_TC_H>(m, a);
+  return gemm(m, m->w3b, m->ld_h, O, m->h2b, m->ld_h, B, H, true, true);
 }
 
 // BF16 operand copies of the FP32 master weights: W1, W2, W3 row-major (padded) and W2^T, W3^T.
 void refresh_bf16(qg_mlp *m) {
   const int H = m->n_h, I = m->n_in, O = m->n_out;
   cudaStream_t s = m->stream;
-  pdl_launch(k_rows_bf16, dim3((I + 255) / 256, std::min(H, 65535)), dim3(256), 0, s, m->w + m->o_w1, I, m->w1b, m->ld_i,
-             H, I);
-  pdl_launch(k_rows_bf16, dim3((H + 255) / 256, std::min(H, 65535)), dim3(256), 0, s, m->w + m->o_w2, H, m->w2b, m->ld_h,
-             H, H);
-  pdl_launch(k_rows_bf16, dim3((H + 255) / 256, std::min(O, 65535)), dim3(256), 0, s, m->w + m->o_w3, H, m->w3b, m->ld_h,
-             O, H);
-  pdl_launch(k_transpose_bf16, dim3((H + 31) / 32, (H + 31) / 32), dim3(32, 8), 0, s, m->w + m->o_w2, H, m->w2t,
-             m->ld_h, H, H);
-  pdl_launch(k_transpose_bf16, dim3((H + 31) / 32, (O + 31) / 32), dim3(32, 8), 0, s, m->w + m->o_w3, H, m->w3t,
-             m->ld_o, O, H);
+  pdl_launch(k_tile_bf16, tiles64(H, I), dim3(256), 0, s, m->w + m->o_w1, m->w1b, m->ld_i, (__nv_bfloat16 *)nullptr, 0LL, H, I);
+  pdl_launch(k_tile_bf16, tiles64(H, H), dim3(256), 0, s, m->w + m->o_w2, m->w2b, m->ld_h, m->w2t, m->ld_h, H, H);
+  pdl_launch(k_tile_bf16, tiles64(O, H), dim3(256), 0, s, m->w + m->o_w3, m->w3b, m->ld_h, m->w3t, m->ld_o, O, H);
 }
 
 }  // namespace
@@ -663,9 +807,8 @@ int qg_mlp_create(qg_mlp **out, int32_t n_in, int32_t n_hidden, int32_t n_out, i
       (rc = mal(m, &m->h1t, H * lb)) || (rc = mal(m, &m->h2b, B * lh)) || (rc = mal(m, &m->h2t, H * lb)) ||
       (rc = mal(m, &m->dyb, B * lo)) || (rc = mal(m, &m->dyt, O * lb)) || (rc = mal(m, &m->dz2b, B * lh)) ||
       (rc = mal(m, &m->dz2t, H * lb)) || (rc = mal(m, &m->dz1t, H * lb)) || (rc = mal(m, &m->z1, B * H)) ||
-      (rc = mal(m, &m->z2, B * H)) || (rc = mal(m, &m->y, B * O)) || (rc = mal(m, &m->dy, B * O)) ||
-      (rc = mal(m, &m->dz2, B * H)) || (rc = mal(m, &m->dz1, B * H)) || (rc = mal(m, &m->part, m->part_elems)) ||
-      (rc = mal(m, &m->lpart, 152 * 8)) || (rc = mal(m, &m->d_err, 1))) {
+      (rc = mal(m, &m->z2, B * H)) || (rc = mal(m, &m->part, m->part_elems)) ||
+      (rc = mal(m, &m->lpart, (O + 31) / 32)) || (rc = mal(m, &m->d_err, 1))) {
     qg_mlp_destroy(m);
     return rc;
   }
@@ -706,10 +849,12 @@ int qg_mlp_set_stream(qg_mlp *m, void *stream) {
 int qg_mlp_forward(qg_mlp *m, const float *x, int32_t batch, float *y) {
   if (!m || !x || !y || batch < 1 || batch > m->max_b) return m ? mfail(m, QG_ERR_INVALID_ARG, "forward arguments") : QG_ERR_INVALID_ARG;
   load_x(m, x, batch, false);
-  int rc = forward(m, batch);
-  if (rc) return rc;
-  cudaError_t e = cudaMemcpyAsync(y, m->y, sizeof(float) * batch * m->n_out, cudaMemcpyDeviceToDevice, m->stream);
-  if (e == cudaSuccess) e = cudaGetLastError();
+  const int sp = forward(m, batch);
+  if (!sp) return QG_ERR_CUDA;
+  EpiArgs a{};
+  a.P = m->part; a.B = batch; a.N = m->n_out; a.splits = sp; a.bias = m->w + m->o_b3; a.Z = y;
+  epi<EPI_OUT, EPI_TC_O>(m, a);
+  cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? QG_OK : mfail(m, QG_ERR_CUDA, cudaGetErrorString(e));
 }
 
@@ -720,38 +865,48 @@ int qg_mlp_train_step(qg_mlp *m, const float *x, const float *target, int32_t ba
   const int B = batch, H = m->n_h, I = m->n_in, O = m->n_out;
   cudaStream_t s = m->stream;
   load_x(m, x, B, true);
-  int rc = forward(m, B);
-  if (rc) return rc;
-  const long long ny = (long long)B * O;
-  const int lb = grid_for(ny);
-  pdl_launch(k_loss, dim3(lb), dim3(256), 0, s, m->y, target, m->dyb, m->ld_o, m->dyt, m->ld_b, m->dy, m->lpart, B,
-             O);
-  if (loss) pdl_launch(k_loss_final, dim3(1), dim3(256), 0, s, m->lpart, lb, ny, loss);
-  // layer 3: dW3 = dY^T H2 (K = the batch: one split, written straight into the gradient),
-  // db3 = colsum(dY), dH2 = dY W3 masked by relu'(Z2)
-  int sp = gemm(m, m->dyt, m->ld_b, O, m->h2t, m->ld_b, H, B, false, false, m->gw + m->o_w3);
+  int sp = forward(m, B);
   if (!sp) return QG_ERR_CUDA;
-  pdl_launch(k_colsum, dim3((O + 255) / 256), dim3(256), 0, s, m->dy, B, O, m->gw + m->o_b3);
+  const long long ny = (long long)B * O;
+  // dY = 2 (Y - target) / (B O), the squared error and db3 = colsum(dY), from the last layer's partials
+  EpiArgs a{};
+  a.P = m->part; a.B = B; a.N = O; a.splits = sp; a.bias = m->w + m->o_b3; a.target = target; a.lpart = m->lpart;
+  a.bgrad = m->gw + m->o_b3; a.Hb = m->dyb; a.ldh = m->ld_o; a.HbT = m->dyt; a.ldt = m->ld_b;
+  epi<EPI_LOSS, EPI_TC_O>(m, a);
+  if (loss)
+    pdl_launch(k_loss_final, dim3(1), dim3(256), 0, s, (const double *)m->lpart, (O + EPI_TC_O - 1) / EPI_TC_O, ny, loss);
+  // layer 3: dW3 = dY^T H2 (K = the batch: one split, written straight into the gradient),
+  // dH2 = dY W3 masked by relu'(Z2), db2 its column sums
+  if (!gemm(m, m->dyt, m->ld_b, O, m->h2t, m->ld_b, H, B, false, false, m->gw + m->o_w3)) return QG_ERR_CUDA;
   if (!(sp = gemm(m, m->w3t, m->ld_o, H, m->dyb, m->ld_o, B, O, true, true))) return QG_ERR_CUDA;
-  pdl_launch(k_bwd_epi, dim3(grid_for((long long)B * H)), dim3(256), 0, s, m->part, sp, m->z2, m->dz2, m->dz2b, m->ld_h,
-             m->dz2t, m->ld_b, B, H);
+  a.N = H; a.splits = sp; a.zmask = m->z2; a.bgrad = m->gw + m->o_b2; a.Hb = m->dz2b; a.ldh = m->ld_h; a.HbT = m->dz2t;
+  epi<EPI_BACK, EPI_TC_H>(m, a);
   // layer 2
-  if (!(sp = gemm(m, m->dz2t, m->ld_b, H, m->h1t, m->ld_b, H, B, false, false, m->gw + m->o_w2))) return QG_ERR_CUDA;
-  pdl_launch(k_colsum, dim3((H + 255) / 256), dim3(256), 0, s, m->dz2, B, H, m->gw + m->o_b2);
+  if (!gemm(m, m->dz2t, m->ld_b, H, m->h1t, m->ld_b, H, B, false, false, m->gw + m->o_w2)) return QG_ERR_CUDA;
   if (!(sp = gemm(m, m->w2t, m->ld_h, H, m->dz2b, m->ld_h, B, H, true, true))) return QG_ERR_CUDA;
-  pdl_launch(k_bwd_epi, dim3(grid_for((long long)B * H)), dim3(256), 0, s, m->part, sp, m->z1, m->dz1, nullptr, 0,
-             m->dz1t, m->ld_b, B, H);
+  a.splits = sp; a.zmask = m->z1; a.bgrad = m->gw + m->o_b1; a.Hb = nullptr; a.HbT = m->dz1t;
+  epi<EPI_BACK, EPI_TC_H>(m, a);
   // layer 1
-  if (!(sp = gemm(m, m->dz1t, m->ld_b, H, m->xt, m->ld_b, I, B, false, false, m->gw + m->o_w1))) return QG_ERR_CUDA;
-  pdl_launch(k_colsum, dim3((H + 255) / 256), dim3(256), 0, s, m->dz1, B, H, m->gw + m->o_b1);
-  // Adam
+  if (!gemm(m, m->dz1t, m->ld_b, H, m->xt, m->ld_b, I, B, false, false, m->gw + m->o_w1)) return QG_ERR_CUDA;
+  // Adam and the BF16 copies of the updated weights
   if (lr > 0) {
     m->step += 1;
-    const double c1 = 1.0 / (1.0 - std::pow(beta1, (double)m->step));
-    const double c2 = 1.0 / (1.0 - std::pow(beta2, (double)m->step));
-    pdl_launch(k_mlp_adam, dim3(grid_for(m->n_par)), dim3(256), 0, s, m->w, m->gw, m->am, m->av, m->n_par, (float)lr,
-               (float)beta1, (float)beta2, (float)c1, (float)c2, 1e-8f);
-    refresh_bf16(m);
+    AdamArgs ad{};
+    const long long rows[3] = {H, H, O}, cols[3] = {I, H, H}, offs[3] = {m->o_w1, m->o_w2, m->o_w3};
+    __nv_bfloat16 *const cb[3] = {m->w1b, m->w2b, m->w3b}, *const ct[3] = {nullptr, m->w2t, m->w3t};
+    const long long ldb[3] = {m->ld_i, m->ld_h, m->ld_h}, ldt[3] = {0, m->ld_h, m->ld_o};
+    for (int q = 0; q < 3; ++q) {
+      const dim3 t = tiles64(rows[q], cols[q]);
+      ad.m[q] = AdamMat{offs[q], (int)rows[q], (int)cols[q], ad.n_tiles, (int)t.x, cb[q], ldb[q], ct[q], ldt[q]};
+      ad.n_tiles += (int)(t.x * t.y);
+    }
+    ad.bias_off[0] = m->o_b1; ad.bias_off[1] = m->o_b2; ad.bias_off[2] = m->o_b3;
+    ad.bias_n[0] = H; ad.bias_n[1] = H; ad.bias_n[2] = O;
+    ad.lr = (float)lr; ad.b1 = (float)beta1; ad.b2 = (float)beta2; ad.eps = 1e-8f;
+    ad.c1 = (float)(1.0 / (1.0 - std::pow(beta1, (double)m->step)));
+    ad.c2 = (float)(1.0 / (1.0 - std::pow(beta2, (double)m->step)));
+    pdl_launch(k_mlp_adam, dim3(ad.n_tiles + (2 * H + O + 255) / 256), dim3(256), 0, s, m->w, (const float *)m->gw, m->am,
+               m->av, ad);
   }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? QG_OK : mfail(m, QG_ERR_CUDA, cudaGetErrorString(e));
