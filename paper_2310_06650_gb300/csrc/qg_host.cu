@@ -12,12 +12,14 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
 
 #include "qg_internal.h"
+#include "qg_split.h"
 #include "qg_sparse.h"
 
 using namespace qg;
@@ -86,6 +88,7 @@ struct qg_ctx {
   std::vector<void *> allocs;
   Dev<double, double> d64{};
   Dev<float, df32> d32{};
+  std::unique_ptr<SplitMat> tail;  // sparse mode: the dense tail's inverse (d64.tail or d32.tail)
   double *d_obj = nullptr, *d_terms = nullptr;
   void *d_g = nullptr, *d_m = nullptr, *d_v = nullptr;
   void *d_xs = nullptr;    // staging for qg_eval_grad_host (Real)
@@ -712,12 +715,7 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
     const int nr = H0.n - 1;
     P.sp_inj_blocks = ceil_div((long long)nr * H0.T, NTHR);
     P.sp_fw_blocks = ceil_div(H0.nS, NTHR / 32) + H0.nT;  // eliminated rows 8 per block, tail rows 1 per block
-    // column splits: about two waves of tail blocks, at least SP_BK columns per split
-    const int n_rt = ceil_div(H0.nT, SP_RB);
-    const int ks0 = n_rt > 0 ? std::max(1, std::min(ceil_div(2 * CTG_WAVE, n_rt), ceil_div(H0.nT, SP_BK))) : 1;
-    P.sp_tail_kc = std::max(SP_BK, ceil_div(ceil_div(H0.nT, ks0), SP_BK) * SP_BK);
-    P.sp_tail_ks = std::max(1, ceil_div(H0.nT, P.sp_tail_kc));
-    P.sp_tail_blocks = n_rt * P.sp_tail_ks;
+    P.sp_tail = H0.nT > 0 ? 1 : 0;
     P.sp_bw_blocks = ceil_div(H0.nS, NTHR / 32);
     P.sp_bwa_blocks = ceil_div((long long)H0.adj_rows.size(), NTHR / 32);
   }
@@ -885,6 +883,40 @@ int upload_selection(qg_ctx *h, int b) {
 }
 
 // Build every device array of one precision flavour.
+void dfree(qg_ctx *h, const void *p);
+
+// S^-1 of the dense tail in digits for the tensor cores (qg_split.h), its buffers and tensor maps.
+template <typename Real, typename Dc>
+int build_tail(qg_ctx *h, Dev<Real, Dc> &d, const HostInst &H) {
+  constexpr int S = split_digits<Dc>();
+  h->tail.reset(new SplitMat{});
+  SplitMat &m = *h->tail;
+  m.rows = m.K = H.nT;
+  m.T = H.T;
+  m.ld = ceil_div(H.nT, 8) * 8;
+  const int passes = ceil_div(H.T, SPLIT_NT);
+  m.nt = ceil_div(ceil_div(H.T, passes), 16) * 16;
+  // one block per SM: each holds the accumulators' tensor memory and nearly all of the shared memory
+  const int n_rt = ceil_div(m.rows, SPLIT_ROWS), nkb = ceil_div(m.K, SPLIT_KB);
+  m.kbps = ceil_div(nkb, std::max(1, std::min(nkb, 152 / n_rt)));
+  m.ks = ceil_div(nkb, m.kbps);
+  int rc;
+  longlong2 *part;
+  if ((rc = dalloc(h, &m.a, (size_t)split_elems(m, S))) || (rc = dalloc(h, &m.b, (size_t)S * m.T * m.ld)) ||
+      (rc = dalloc(h, &m.ascale, (size_t)m.rows)) || (rc = dalloc(h, &m.bscale, (size_t)m.T)) ||
+      (rc = dalloc(h, &part, (size_t)m.ks * n_rt * SPLIT_ROWS * m.T)))
+    return rc;
+  m.part = part;
+  d.tail = &m;
+  if (!split_maps(m, S)) return fail(h, QG_ERR_UNSUPPORTED, "the driver's TMA descriptor encoder is not available");
+  double *src;
+  if ((rc = upload(h, &src, H.sinv))) return rc;
+  CUDA_TRY(h, split_matrix(m, src, S, h->stream));
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  dfree(h, src);
+  return QG_OK;
+}
+
 template <typename Real, typename Dc>
 int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) {
   const int B = h->n_inst;
@@ -1141,7 +1173,7 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
     UPI(bus_pos, H.bus_pos) UPI(pos_gb, H.pos_gb) UPI(pos_bus, H.pos_bus) UPI(fw_ptr, H.fw_ptr) UPI(fw_col, H.fw_col)
     UPI(bw_ptr, H.bw_ptr) UPI(bw_col, H.bw_col) UPI(adj_rows, H.adj_rows) UPI(inc_ptr, H.inc_ptr)
     UPI(inc_code, H.inc_code)
-    UPD(fw_val, H.fw_val) UPD(bw_val, H.bw_val) UPD(dinv, H.dinv) UPD(sinv, H.sinv) UPD(z1, H.z1) UPD(ydc, ydc)
+    UPD(fw_val, H.fw_val) UPD(bw_val, H.bw_val) UPD(dinv, H.dinv) UPD(z1, H.z1) UPD(ydc, ydc)
     UPD(load_dc, H.load_p)
 #undef UPI
 #undef UPD
@@ -1159,11 +1191,10 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
     d.sp_mu = c;
     if ((rc = dalloc(h, &c, (size_t)d.n_pchunk * H.T))) return rc;
     d.sp_part = c;
-    if ((rc = dalloc(h, &c, (size_t)std::max(1LL, (long long)P.sp_tail_ks * d.nT * H.T)))) return rc;
-    d.sp_tpart = c;
     unsigned int *tk;
-    if ((rc = dalloc(h, &tk, (size_t)std::max(1, ceil_div(d.nT, SP_RB))))) return rc;
-    d.sp_tick = tk;
+    if ((rc = dalloc(h, &tk, (size_t)2 * SPLIT_SPREAD * H.T))) return rc;
+    d.sp_bmax = tk;
+    if (d.nT > 0 && (rc = build_tail(h, d, H))) return rc;
   }
   const qg_options &o = h->opt;
   d.c_p = (Real)o.c_p; d.c_q = (Real)o.c_q; d.c_s = (Real)o.c_s; d.c_rz = (Real)o.c_rz;
@@ -2243,7 +2274,7 @@ int32_t qg_launches_per_eval(const qg_ctx *h) {
   const int s2 = P.s2.n_blocks > 0 ? 1 + (P.ctg_lazy ? 1 : 0) : 0;
   // + 1: the closing kernel (the mixed path's dense mode updates the devices in stage 4)
   if (!P.sp) return 3 + s2 + (P.s5.n_blocks > 0 ? 1 : 0) + 1;
-  return 4 + s2 + 3 + (P.sp_tail_blocks > 0 ? 2 : 0) + (P.sp_bw_blocks > 0 ? 1 : 0) + (P.sp_bwa_blocks > 0 ? 1 : 0) + 1;
+  return 4 + s2 + 3 + (P.sp_tail ? 6 : 0) + (P.sp_bw_blocks > 0 ? 1 : 0) + (P.sp_bwa_blocks > 0 ? 1 : 0) + 1;
 }
 
 int32_t qg_ctg_path(const qg_ctx *h) {

@@ -94,9 +94,6 @@ struct Inst {
 // the adjoint solve), whose device updates are R_GEN / R_XF blocks of stage 5.
 enum Role : int { R_BRANCH = 0, R_ZONE, R_DCF, R_BUS, R_CTG, R_GBUS, R_GEN, R_SDCF, R_SDCA, R_XF, R_OBJ, R_HOT };
 
-constexpr int SP_RB = 64;   // dense tail product: rows per block
-constexpr int SP_BK = 32;   // dense tail product: columns per shared-memory chunk
-constexpr int SP_TMAX = 48; // periods per pass of the dense tail product (16 lanes x 3)
 
 // A run of blocks with one role for one instance: blocks [first, first + per_t * nt);
 // block b of the span has period (or period chunk) (b - first) / per_t and slice (b - first) % per_t.
@@ -122,6 +119,8 @@ struct InstTab {
 struct df32 {
   float hi, lo;
 };
+
+struct SplitMat;  // qg_split.h
 
 // Device arrays.  Real is double (QG_FP64) or float (QG_MIXED); Dc is the DC
 // product type: double, or df32 in the mixed path.
@@ -186,15 +185,14 @@ struct Dev {
   const Dc *bw_val;
   const int *adj_rows;                // [n_adj_rows]
   const Dc *dinv;                     // [nS] 1 / D_S
-  const Dc *sinv;                     // [nT nT] S^-1, row-major
+  const SplitMat *tail;               // host only: S^-1 in digits (NULL without a tail)
   const Dc *z1;                       // [nr] Yhat^-1 1 at each position
   const int *inc_ptr, *inc_code;      // position -> incident branches, code = j << 1 | (1 at the to-end)
   const Dc *ydc;                      // [M] y_j = -b_sr
   Dc *sp_rhs, *sp_u, *sp_th, *sp_zt;  // [nr T], [nr T], [nr T], [nT T]
   Dc *sp_mu;                          // [T] mean injection (uniform slack)
   Dc *sp_part;                        // [n_pchunk][T] partial sums of z1 . w
-  Dc *sp_tpart;                       // [tail splits][nT][T] partial sums of the dense tail product
-  unsigned int *sp_tick;              // [tail row tiles] last-split tickets (zero between launches)
+  unsigned int *sp_bmax;              // [2][SPLIT_SPREAD][T] largest |z_T| per period, forward and adjoint solve (bits)
   // penalty parameters
   Real c_p, c_q, c_s, c_rz, rho, eps, beta;
   double c_s64, eps64, beta64;        // the same options in FP64 (closed-form objective floor)
@@ -259,9 +257,7 @@ struct Plan {
   int sp;
   int sp_inj_blocks;   // right-hand-side blocks of k_sp_inj (T more compute the mean injection)
   int sp_fw_blocks;    // k_sp_fwd rows / 8
-  int sp_tail_blocks;  // k_sp_tail, 0 without a tail
-  int sp_tail_ks;      // column splits of the dense tail product
-  int sp_tail_kc;      // columns per split (a multiple of SP_BK)
+  int sp_tail;         // 1: a dense tail (its product takes three kernels)
   int sp_bw_blocks;    // k_sp_back forward pass
   int sp_bwa_blocks;   // k_sp_back adjoint pass
 };

@@ -19,7 +19,7 @@
 //       incl. the slack-corrected injection adjoint eta - mean(eta) (Eq.
 //       correction) [+ fused Adam] | transformer gradients; the last block
 //       reduces the objective and advances the Adam step counter.
-// Sparse DC mode: k_sp_inj, k_sp_fwd, k_sp_tail, k_sp_back solve Yhat theta = b
+// Sparse DC mode: k_sp_inj, k_sp_fwd, the tail product (qg_split.cu), k_sp_back solve Yhat theta = b
 // through the sparse factor with a dense tail, before s1 and after s4.
 // No floating-point atomics: every sum has a fixed order, so repeated
 // evaluations are bitwise identical.
@@ -36,6 +36,7 @@
 #include <vector>
 
 #include "qg_internal.h"
+#include "qg_split.h"
 
 namespace qg {
 
@@ -191,6 +192,9 @@ struct DcOps<df32> {
   __device__ static df32 bcast(df32 a) { return {__shfl_sync(0xffffffffu, a.hi, 0), __shfl_sync(0xffffffffu, a.lo, 0)}; }
 };
 
+// |a| rounded up to FP32
+__device__ __forceinline__ float abs_up(double a) { return __double2float_ru(fabs(a)); }
+__device__ __forceinline__ float abs_up(df32 a) { return __fadd_ru(fabsf(a.hi), fabsf(a.lo)); }
 __device__ __forceinline__ double to_double(double a) { return a; }
 __device__ __forceinline__ double to_double(df32 a) { return (double)a.hi + (double)a.lo; }
 
@@ -2639,6 +2643,7 @@ __global__ void __launch_bounds__(NTHR) k_sp_inj(const __grid_constant__ Dev<Rea
     d.sp_rhs[e] = s;
   } else {
     const int t = blockIdx.x - nb;
+    if ((int)threadIdx.x < 2 * SPLIT_SPREAD) d.sp_bmax[threadIdx.x * I.T + t] = 0u;  // of both solves of this evaluation
     Dc s = DcOps<Dc>::zero();
     for (int g = threadIdx.x; g < I.G; g += NTHR)
       s = DcOps<Dc>::add(s, DcOps<Dc>::from_real(d.gen_sgn[I.gen0 + g] * p[(long long)t * I.G + g]));
@@ -2710,97 +2715,21 @@ __global__ void __launch_bounds__(NTHR) k_sp_fwd(const __grid_constant__ Dev<Rea
         }
         const Dc *b = d.sp_rhs + (long long)row * T;
         Dc *z = d.sp_zt + (long long)(row - d.nS) * T;
-        if (ta < T) z[ta] = DcOps<Dc>::add(b[ta], z0);
-        if (tb < T) z[tb] = DcOps<Dc>::add(b[tb], z1);
+        // the running maxima of |z_T| per period scale the tail product's digits (a maximum: the same in
+        // any order; SPLIT_SPREAD copies, so that few rows meet at one address)
+        unsigned *mx = d.sp_bmax + ((ADJ ? SPLIT_SPREAD : 0) + row % SPLIT_SPREAD) * T;
+        if (ta < T) {
+          z[ta] = z0 = DcOps<Dc>::add(b[ta], z0);
+          atomicMax(mx + ta, __float_as_uint(abs_up(z0)));
+        }
+        if (tb < T) {
+          z[tb] = z1 = DcOps<Dc>::add(b[tb], z1);
+          atomicMax(mx + tb, __float_as_uint(abs_up(z1)));
+        }
       }
       __syncthreads();
     }
   }
-}
-
-// Dense tail x_T = S^-1 z_T (a dense contraction, but in double-FP32 for the FP64-accurate DC
-// solve, so on the FP32 pipes).  Block (row tile, column split): SP_RB rows x the split's share of
-// the columns x all periods (up to SP_TMAX per pass); thread (row group, period lane) holds 4 rows
-// x 4 periods of accumulators; S^-1 and z_T staged through shared memory SP_BK columns at a time.
-// Each split writes its partial sums; the last split of a row tile to finish (ticket) adds them in
-// split order and writes u (for the backward gather) and the solution (forward pass) or the
-// generator-bus adjoints (adjoint pass).
-template <typename Real, typename Dc, bool ADJ>
-__global__ void __launch_bounds__(NTHR, 2) k_sp_tail(const __grid_constant__ Dev<Real, Dc> d,
-                                                  const __grid_constant__ Inst I, int ks, int kchunk) {
-  __shared__ Dc s_s[SP_RB][SP_BK + 1];
-  __shared__ Dc s_z[SP_BK][SP_TMAX];
-  __shared__ bool last;
-  const int T = I.T, m = d.nT;
-  const int rt = blockIdx.x / ks, kp = blockIdx.x % ks;
-  const int a0 = rt * SP_RB;
-  const int b_lo = min(m, kp * kchunk), b_hi = min(m, b_lo + kchunk);
-  const int rg = threadIdx.x >> 4, tc = threadIdx.x & 15;
-  pdl_wait();
-  for (int t0 = 0; t0 < T; t0 += SP_TMAX) {
-    const int tn = min(SP_TMAX, T - t0);
-    Dc acc[4][SP_TMAX / 16];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < SP_TMAX / 16; ++j) acc[i][j] = DcOps<Dc>::zero();
-    for (int b0 = b_lo; b0 < b_hi; b0 += SP_BK) {
-      const int bn = min(SP_BK, b_hi - b0);
-      __syncthreads();
-#pragma unroll
-      for (int e = threadIdx.x; e < SP_RB * SP_BK; e += NTHR) {
-        const int rr = e / SP_BK, cc = e % SP_BK, ar = a0 + rr;
-        s_s[rr][cc] = (ar < m && cc < bn) ? d.sinv[(long long)ar * m + b0 + cc] : DcOps<Dc>::zero();
-      }
-#pragma unroll
-      for (int e = threadIdx.x; e < SP_BK * SP_TMAX; e += NTHR) {
-        const int rr = e / SP_TMAX, cc = e % SP_TMAX;
-        s_z[rr][cc] = (rr < bn && cc < tn) ? d.sp_zt[(long long)(b0 + rr) * T + t0 + cc] : DcOps<Dc>::zero();
-      }
-      __syncthreads();
-#pragma unroll 2
-      for (int k = 0; k < SP_BK; ++k) {
-        Dc sv[4], zv[SP_TMAX / 16];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) sv[i] = s_s[rg * 4 + i][k];
-#pragma unroll
-        for (int j = 0; j < SP_TMAX / 16; ++j) zv[j] = s_z[k][tc + 16 * j];
-#pragma unroll
-        for (int j = 0; j < SP_TMAX / 16; ++j)
-          if (tc + 16 * j < tn)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) DcOps<Dc>::mac(acc[i][j], sv[i], zv[j]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int a = a0 + rg * 4 + i;
-      if (a >= m) continue;
-#pragma unroll
-      for (int j = 0; j < SP_TMAX / 16; ++j)
-        if (tc + 16 * j < tn) d.sp_tpart[((long long)kp * m + a) * T + t0 + tc + 16 * j] = acc[i][j];
-    }
-  }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(d.sp_tick + rt, 1u) == (unsigned)(ks - 1);
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  for (int e = threadIdx.x; e < SP_RB * T; e += NTHR) {
-    const int a = a0 + e / T, t = e % T;
-    if (a >= m) continue;
-    Dc v = DcOps<Dc>::zero();
-    for (int q = 0; q < ks; ++q) v = DcOps<Dc>::add(v, d.sp_tpart[((long long)q * m + a) * T + t]);
-    const int pos = d.nS + a;
-    d.sp_u[(long long)pos * T + t] = v;
-    d.sp_th[(long long)pos * T + t] = v;  // forward: the angles; adjoint: eta (transformer gradients)
-    if (ADJ) {
-      const int gb = d.pos_gb[pos];
-      if (gb >= 0) d.gip[I.gi0 + (long long)t * (I.Gc + 1) + gb] = v;
-    }
-  }
-  if (threadIdx.x == 0) d.sp_tick[rt] = 0u;
 }
 
 // Backward gather x_S = M1^T u_S + M2^T u_T (u_S = D_S^-1 z_S, u_T = x_T), one warp per eliminated
@@ -2916,6 +2845,16 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
       e = cudaGetLastError();
     }
   };
+  // dense tail x_T = S^-1 z_T of a sparse solve
+  auto tail = [&](bool adj, const Inst &I) {
+    if (!P.sp_tail || e != cudaSuccess) return;
+    SplitMat m = *d.tail;
+    m.bmax = d.sp_bmax + (adj ? SPLIT_SPREAD * I.T : 0);
+    e = split_rhs<Dc>(m, d.sp_zt, s, pdl);
+    if (e == cudaSuccess)
+      e = split_product<Dc>(m, SplitOut<Dc>{d.sp_u, d.sp_th, d.nS, adj ? d.pos_gb : nullptr,
+                                            d.gip + I.gi0, I.Gc + 1}, s, pdl);
+  };
   mark(ev, 0, s);
   nvtxRangePushA("qg stage 1");  // one NVTX range per stage, closed at the next stage's launch
   if (P.sp) {
@@ -2924,7 +2863,7 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
     k_sp_inj<Real, Dc><<<P.sp_inj_blocks + I.T, NTHR, 0, s>>>(d, I, (const Real *)x, P.sp_inj_blocks);
     e = cudaGetLastError();
     go(k_sp_fwd<Real, Dc, false>, P.sp_fw_blocks, 0, d, I, P.sp_fw_blocks);
-    if (P.sp_tail_blocks > 0) go(k_sp_tail<Real, Dc, false>, P.sp_tail_blocks, 0, d, I, P.sp_tail_ks, P.sp_tail_kc);
+    tail(false, I);
     if (P.sp_bw_blocks > 0) go(k_sp_back<Real, Dc, false>, P.sp_bw_blocks, 0, d, I);
     go(k_s1<Real, Dc>, P.s1.n_blocks, 0, d, P.tab, P.s1, (const Real *)x, 0);
   } else {
@@ -2962,7 +2901,7 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
     // sparse mode: adjoint solve eta = Yhat^-1 w at the generator buses, and 1^T eta
     const Inst &I = P.tab.I[0];
     go(k_sp_fwd<Real, Dc, true>, P.sp_fw_blocks + (I.T + NTHR / 32 - 1) / (NTHR / 32), 0, d, I, P.sp_fw_blocks);
-    if (P.sp_tail_blocks > 0) go(k_sp_tail<Real, Dc, true>, P.sp_tail_blocks, 0, d, I, P.sp_tail_ks, P.sp_tail_kc);
+    tail(true, I);
     if (P.sp_bwa_blocks > 0) go(k_sp_back<Real, Dc, true>, P.sp_bwa_blocks, 0, d, I);
   }
   mark(ev, 4, s);

@@ -71,11 +71,14 @@ __device__ __forceinline__ bool mbar_test(uint64_t *b, uint32_t parity) {
 // or at once when another thread of the block has given up (abort != 0 and honour_abort); returns
 // whether the phase completed.
 __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, volatile int *abort, bool honour_abort) {
+  // the clock is read only once the first polls have failed: reading it costs more than a met wait
+  for (int it = 0; it < 16; ++it)
+    if (mbar_test(b, parity)) return true;
   const unsigned long long t0 = gtime();
   for (unsigned it = 0; it < (1u << 30); ++it) {
     if (mbar_test(b, parity)) return true;
     if (honour_abort && *abort) return false;
-    if (gtime() - t0 > WAIT_NS) break;
+    if ((it & 15) == 15 && gtime() - t0 > WAIT_NS) break;
   }
   *abort = 1;
   return false;
