@@ -101,18 +101,26 @@ struct Span {
   int first, per_t, nt, inst, role;
 };
 
-struct Spans {
-  Span s[MAXSPAN];
+// The span and instance tables travel as kernel parameters, in two sizes: of the whole batch, and of a
+// handle with one instance (NI = 1), whose launches then carry 1.5 KB of parameters instead of 17 KB.
+constexpr int ONE_SPANS = 6;  // spans of a launch of one instance (at most one per role)
+
+template <int NI>
+struct SpansT {
+  Span s[NI == 1 ? ONE_SPANS : MAXSPAN];
   int n;
   int n_blocks;
 };
+using Spans = SpansT<MAXB>;
 
-struct InstTab {
-  Inst I[MAXB];
+template <int NI>
+struct InstTabT {
+  Inst I[NI];
   int n_inst;
   int fuse;  // 1: stage 4's warps update the devices (the last stage); 0: stage 5 does
   int s3q;   // threads per branch-period in stage 3 (1 or S3_SPLIT_MAX; the kernel's template argument)
 };
+using InstTab = InstTabT<MAXB>;
 
 // Double-FP32 value (unevaluated sum hi + lo) carrying the FP64-accurate DC
 // products of the mixed path: GB300's FP64 pipe runs at ~1/60 of its FP32 rate.
@@ -210,7 +218,7 @@ struct Dev {
   Real *dZ;                           // [sum T Z]
   Real *pm, *pq, *pk;                 // contingency partials
   unsigned char *hot;                 // [sum T M] 1: a hot row (its partials are s2_hot's)
-  Real *pkh, *pzh;                    // column (score) partials of the hot rows, [hot][T][Kp] per instance (pkh without the period's weight)
+  Real *pkh, *pzh;                    // column (score) partials of the hot rows, [hot][T][Kp] per instance
   unsigned char *pmf;                 // row-partial flags (pm, pq are written and read only where set)
   int score;                          // 1: record per-(period, outage) scores (contingency screening)
   Real *pz;                           // score partials [n_mg][T][K] per instance (at pk0)

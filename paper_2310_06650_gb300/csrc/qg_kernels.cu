@@ -229,6 +229,11 @@ __device__ __forceinline__ void root_and_ratio(Real a, Real w, Real &s, Real &q)
   }
 }
 
+// a^2 + b^2, the FP32 form with its multiply-add spelled out (the bits of the adjoints do not hang on how the
+// compiler contracts it)
+__device__ __forceinline__ double sq_sum(double a, double b) { return a * a + b * b; }
+__device__ __forceinline__ float sq_sum(float a, float b) { return __fmaf_rn(a, a, __fmul_rn(b, b)); }
+
 // soft-ReLU sigma_s(u) = sqrt(max(u,0)^2 + eps^2) and its derivative max(u,0) / sigma_s(u)
 // (Sec. II-C footnote)
 template <typename Real>
@@ -400,7 +405,8 @@ __device__ __forceinline__ HP<Real> hparams(const Dev<Real, Dc> &d) {
 }
 
 // Block -> (role, instance, period or period chunk, slice) by binary search over the spans.
-__device__ __forceinline__ Where locate(const Spans &S) {
+template <int NI>
+__device__ __forceinline__ Where locate(const SpansT<NI> &S) {
   const int bid = blockIdx.x;
   int lo = 0, hi = S.n - 1;
   while (lo < hi) {
@@ -745,12 +751,12 @@ __device__ void s1_bus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, co
   }
 }
 
-template <typename Real, typename Dc>
+template <typename Real, typename Dc, int NI>
 __global__ void __launch_bounds__(NTHR) k_s1(const __grid_constant__ Dev<Real, Dc> d,
-                                             const __grid_constant__ InstTab tab, const __grid_constant__ Spans S,
+                                             const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              const Real *__restrict__ x, int slot0) {
   const Where w = locate(S);
-  const Inst &I = tab.I[tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
+  const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
   const int slot = d.slot_map[slot0 + blockIdx.x];  // issued first: it is not needed until the end
   Obj3<Dc> acc = obj3<Dc>(-1);
   if (w.role == R_DCF) {
@@ -894,9 +900,9 @@ constexpr int CT_TBATCH = 12;  // tiles per batch of bound tests on the on-deman
 // smallest clear_margin of the branch over the chunk's periods (FLT_MAX on the pad rows of the last
 // 64-row tile), from the FP32 values the stage-2 screen reads.  Once per evaluation, instead of once
 // per outage tile.
-template <typename Real, typename Dc>
+template <typename Real, typename Dc, int NI>
 __global__ void __launch_bounds__(NTHR) k_ctg_margin(const __grid_constant__ Dev<Real, Dc> d,
-                                                     const __grid_constant__ InstTab tab) {
+                                                     const __grid_constant__ InstTabT<NI> tab) {
   pdl_wait();
   for (int b = 0; b < tab.n_inst; ++b) {
     const Inst &I = tab.I[b];
@@ -1314,22 +1320,32 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
                 if (!(F64 ? y[i][j] >= 0.f : y[i][j] > 0.f)) continue;  // NaN (pad, outaged branch) fails too
                 const Real q2 = d.qm2[I.tm0 + (long long)(t0 + tl) * I.M + m0 + mm];
                 Real Fx, Lx, dd;
-                Real val;
                 if (F64) {
                   Lx = (Real)d.lodf64[I.l0 + (long long)(m0 + mm) * I.Kp + kc + j];
                   Fx = s_f64m[tl * CT_BM + mm] + Lx * s_f64k[tl * CT_BK + cq * 4 + j];
                   const Real a2 = Fx * Fx + q2;
                   if (a2 - s_s2[mm] <= Real(0)) continue;
+                  Real val;
                   ctg_element(a2, s_s2[CT_BM + mm], eps, w, val, dd);
+                  obj += w * (val - eps);
+                  zc[j] += w * (val - eps);
                 } else {
+                  // mixed path: s = sqrt(F^2 + qmax2) and the soft-ReLU through reciprocal square
+                  // roots (a few units in the last place, below the FP32 error of F itself)
                   float l0, l1;
                   unpack2(Lp[i >> 1][j], l0, l1);
                   Lx = (i & 1) ? l1 : l0;
                   Fx = F[i][j];
-                  ctg_element(Real(__fmaf_rn(F[i][j], F[i][j], (float)q2)), s_s2[CT_BM + mm], eps, w, val, dd);
+                  const float a2 = __fmaf_rn(F[i][j], F[i][j], (float)q2);
+                  const float ra = rsqrtf(a2);
+                  const float u = fmaxf(__fmaf_rn(a2, ra, -(float)s_s2[CT_BM + mm]), 0.f);
+                  const float b2 = __fmaf_rn(u, u, (float)(eps * eps));
+                  const float rb = rsqrtf(b2);
+                  const float val = b2 * rb;  // sqrt(u^2 + eps^2)
+                  obj += w * (val - eps);
+                  zc[j] += w * (val - eps);
+                  dd = w * (u * rb) * ra;  // w sigma'(s - s_ctg) / s
                 }
-                obj += w * (val - eps);
-                zc[j] += w * (val - eps);
                 gm[i] += dd * Fx;
                 gk[j] += dd * Fx * Lx;
                 gq[i] += Real(0.5) * dd;     // dz/dqmax2 = w sigma' / (2 s)
@@ -1440,7 +1456,7 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
 // per thread: no idle lanes, no branch per element, the next row's loads in flight while the current one
 // is evaluated.  A row's sums go to its partial slot of the chunk's first outage tile (which the screen
 // leaves to this path), the column sums stay with their thread (in registers while the period lasts,
-// else in pkh, one owner per entry; without the period's weight, which stage 3 applies).  On the mixed path
+// else in pkh, one owner per entry; the period's weight is applied once, at the end).  On the mixed path
 // the block covers what a contingency block covers and sums the objective per row quad and column quad in
 // the screen's order, so that its FP32 rounding stays that of one running sum per thread of such a block.
 constexpr int HOT_MASKS = 32;     // (tile, period) pairs per list
@@ -1678,7 +1694,16 @@ __device__ void s2_hot(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
       __syncthreads();
     }
   }
-  if (col && tcur >= 0) store4(pk + (long long)tcur * I.Kp, gk);
+  if (col) {  // the column sums' weight, once per entry
+    if (tcur >= 0) store4(pk + (long long)tcur * I.Kp, gk);
+    for (int tt = 0; tt < TB; ++tt) {
+      const Real w = d.dt[I.tp0 + t0 + tt] * d.c_s * hp.beta;
+      load4(pk + (long long)tt * I.Kp, gk);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) gk[j] *= w;
+      store4(pk + (long long)tt * I.Kp, gk);
+    }
+  }
   if (F64) {
     acc.v[0] = DcOps<Dc>::from_real(obj);
   } else {
@@ -1689,12 +1714,12 @@ __device__ void s2_hot(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
   }
 }
 
-template <typename Real, typename Dc, int MODE>
+template <typename Real, typename Dc, int MODE, int NI>
 __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s2(const __grid_constant__ Dev<Real, Dc> d,
-                                             const __grid_constant__ InstTab tab, const __grid_constant__ Spans S,
+                                             const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              const Real *__restrict__ x, int slot0) {
   const Where w = locate(S);
-  const Inst &I = tab.I[tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
+  const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
   Obj3<Dc> acc = obj3<Dc>(-1);
   if (w.role == R_BUS) {  // FP64 path
     acc.id[0] = T_ZP;
@@ -1766,12 +1791,12 @@ __device__ void fold_slots(const Dev<Real, Dc> &d, const Inst &I, int r) {
   }
 }
 
-template <typename Real, typename Dc, int SPLIT>
+template <typename Real, typename Dc, int SPLIT, int NI>
 __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __grid_constant__ Dev<Real, Dc> d,
-                                             const __grid_constant__ InstTab tab, const __grid_constant__ Spans S,
+                                             const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              const Real *__restrict__ x) {
   const Where w = locate(S);
-  const Inst &I = tab.I[tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
+  const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
   if (w.role == R_OBJ) {  // whole block
     pdl_wait();
     fold_slots(d, I, w.sub);
@@ -1822,7 +1847,6 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       phi = x[I.xtau0 + (long long)(I.T + t) * I.X + xi0];
     }
   }
-  const Real wctg = d.dt[I.tp0 + t] * d.c_s * hparams(d).beta;  // the hot rows' column sums come without it
   Real gF = 0, gq2 = 0, gk = 0, gh = 0, zk = 0;  // gh: the hot rows' share of gk
   // row partials of the outage tiles whose 64-row tile had an overload (flagged by stage 2), or, for a hot
   // row, of the first outage tile of each of s2_hot's chunks: few tiles are read unconditionally and
@@ -1863,7 +1887,7 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       }
     }
     if (kx >= 0) {
-      if (SPLIT > 1 || I.n_mg + I.hot <= 32) {
+      if (SPLIT > 1 || !I.hot) {
 #pragma unroll 8
         for (int mg = q; mg < I.n_mg; mg += SPLIT) gk += d.pk[I.pk0 + ((long long)mg * I.T + t) * I.K + kx];
 #pragma unroll 8
@@ -1875,7 +1899,7 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       }
     }
   }
-  if (SPLIT == 1 && I.n_mg + I.hot > 32) {
+  if (SPLIT == 1 && I.hot) {
     // many column partials (large plans, where few branches are outages): the whole warp sums those of
     // each of its outage branches, a lane every 32nd, instead of one lane walking them all
     const int lane = threadIdx.x & 31;
@@ -1885,13 +1909,13 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
 #pragma unroll 2
       for (int mg = lane; mg < I.n_mg; mg += 32) s += d.pk[I.pk0 + ((long long)mg * I.T + t) * I.K + k];
 #pragma unroll 4
-      for (int mg = lane; mg < I.hot; mg += 32) s += wctg * d.pkh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + k];
+      for (int mg = lane; mg < I.hot; mg += 32) s += d.pkh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + k];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (lane == src) gk = s;
     }
   }
-  gk += gh * wctg;
+  gk += gh;
 #pragma unroll
   for (int o = 1; o < SPLIT; o <<= 1) {
     gF += __shfl_xor_sync(0xffffffffu, gF, o);
@@ -1902,13 +1926,14 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
   gF += gk;
   if (lead) {
     // adjoints of the four end flows
-    const Real sf2 = pf * pf + qf * qf, st2 = pt * pt + qt * qt;
+    const Real sf2 = sq_sum(pf, qf), st2 = sq_sum(pt, qt);
     if (fmax(sf2, st2) > smax * smax) {  // thermal (Example 1)
       const Real sf = dsqrt(sf2), st = dsqrt(st2);
       const bool fr = sf >= st;
       Real val, der;
       const HP<Real> hp = hparams(d);
-      soft_relu((fr ? sf : st) - smax, hp.eps, val, der);
+      const Real over = fmax((fr ? sf : st) - smax, Real(0));
+      root_and_ratio(sq_sum(over, hp.eps), over, val, der);  // soft-ReLU
       const Real k = d.dt[I.tp0 + t] * d.c_s * hp.beta * der / (fr ? sf : st);
       if (fr) {
         gpf += k * pf;
@@ -2074,8 +2099,8 @@ __device__ void s4_bus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, Re
 // Objective reduction, level 2, run by the closing kernel: per instance, the slots of its
 // device blocks and of its fold blocks in fixed order (read through L2: other blocks wrote them),
 // plus the closed-form soft-ReLU floor of the contingency term.
-template <typename Real, typename Dc>
-__device__ void final_reduce(const Dev<Real, Dc> &d, const InstTab &tab) {
+template <typename Real, typename Dc, int NI>
+__device__ void final_reduce(const Dev<Real, Dc> &d, const InstTabT<NI> &tab) {
   for (int b = 0; b < tab.n_inst; ++b) {
     const Inst &I = tab.I[b];
     Dc a[N_TERMS];
@@ -2406,12 +2431,12 @@ __device__ void s5_xf(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, Rea
 // Stage 5 (sparse DC mode, and the FP64 path's dense mode): devices of one period, with eta from the
 // adjoint solve or from stage 4's products (whose columns already subtract the mean) | transformers
 // of one period; the last block reduces the objective.
-template <typename Real, typename Dc, bool ADAM>
+template <typename Real, typename Dc, bool ADAM, int NI>
 __global__ void __launch_bounds__(NTHR) k_s5(const __grid_constant__ Dev<Real, Dc> d,
-                                             const __grid_constant__ InstTab tab, const __grid_constant__ Spans S,
+                                             const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              Real *__restrict__ x) {
   const Where w = locate(S);
-  const Inst &I = tab.I[tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
+  const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
   const int t = w.t;
   AdamCoef<Real> ac{};
   if (ADAM) ac = adam_coef(d);
@@ -2557,12 +2582,12 @@ __device__ void s4_gbus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, c
 // dense DC mode also the adjoint DC products with the device and transformer updates (the last
 // stage: its last block reduces the objective); in the sparse mode the right-hand side of the
 // adjoint solve.
-template <typename Real, typename Dc, bool ADAM, bool FUSE>
+template <typename Real, typename Dc, bool ADAM, bool FUSE, int NI>
 __global__ void __launch_bounds__(NTHR) k_s4(const __grid_constant__ Dev<Real, Dc> d,
-                                             const __grid_constant__ InstTab tab, const __grid_constant__ Spans S,
+                                             const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              Real *__restrict__ x) {
   const Where w = locate(S);
-  const Inst &I = tab.I[tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
+  const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
   AdamCoef<Real> ac{};
   if (ADAM) ac = adam_coef(d);
   if (w.role == R_BUS) {
@@ -2815,23 +2840,52 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), int grid, size_t smem, cud
 // Closing kernel of an evaluation, or of a graph of n fused iterations: one block sums the
 // objective of the last one from the slots the stage kernels left, then step += n (n = 0 for a
 // plain evaluation).
-template <typename Real, typename Dc>
+template <typename Real, typename Dc, int NI>
 __global__ void __launch_bounds__(NTHR) k_finish(const __grid_constant__ Dev<Real, Dc> d,
-                                                 const __grid_constant__ InstTab tab, int n) {
+                                                 const __grid_constant__ InstTabT<NI> tab, int n) {
   const long long step = *d.step;  // no stage kernel writes it
   pdl_wait();
   final_reduce(d, tab);
   if (threadIdx.x == 0) *d.step = step + n;
 }
 
-template <typename Real, typename Dc>
-cudaError_t launch_finish(const Dev<Real, Dc> &d, const Plan &P, int n, cudaStream_t s) {
-  return launch_pdl(k_finish<Real, Dc>, 1, 0, s, d, P.tab, n);
+// The tables of a plan as the kernels of NI instances take them.
+template <int NI>
+static InstTabT<NI> table(const InstTab &t) {
+  if constexpr (NI == MAXB) return t;
+  else {
+    InstTabT<NI> r;
+    for (int b = 0; b < NI; ++b) r.I[b] = t.I[b];
+    r.n_inst = t.n_inst;
+    r.fuse = t.fuse;
+    r.s3q = t.s3q;
+    return r;
+  }
+}
+template <int NI>
+static SpansT<NI> spans(const Spans &t) {
+  if constexpr (NI == MAXB) return t;
+  else {
+    SpansT<NI> r;
+    for (int k = 0; k < ONE_SPANS; ++k) r.s[k] = t.s[k];
+    r.n = t.n;
+    r.n_blocks = t.n_blocks;
+    return r;
+  }
 }
 
 template <typename Real, typename Dc>
-cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, bool adam, bool close,
-                        cudaStream_t s, cudaEvent_t *ev) {
+cudaError_t launch_finish(const Dev<Real, Dc> &d, const Plan &P, int n, cudaStream_t s) {
+  if (P.tab.n_inst == 1) return launch_pdl(k_finish<Real, Dc, 1>, 1, 0, s, d, table<1>(P.tab), n);
+  return launch_pdl(k_finish<Real, Dc, MAXB>, 1, 0, s, d, P.tab, n);
+}
+
+template <typename Real, typename Dc, int NI>
+static cudaError_t launch_stages(const Dev<Real, Dc> &d, const Plan &P, const void *xv, bool adam, bool close,
+                                 cudaStream_t s, cudaEvent_t *ev) {
+  const InstTabT<NI> tab = table<NI>(P.tab);
+  const SpansT<NI> sp1 = spans<NI>(P.s1), sp2 = spans<NI>(P.s2), sp3 = spans<NI>(P.s3), sp4 = spans<NI>(P.s4),
+                   sp5 = spans<NI>(P.s5);
   Real *x = const_cast<Real *>(static_cast<const Real *>(xv));
   const int o2 = P.s1.n_blocks;
   // with timing events between the kernels, launch them plainly so each event brackets one kernel
@@ -2865,37 +2919,37 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
     go(k_sp_fwd<Real, Dc, false>, P.sp_fw_blocks, 0, d, I, P.sp_fw_blocks);
     tail(false, I);
     if (P.sp_bw_blocks > 0) go(k_sp_back<Real, Dc, false>, P.sp_bw_blocks, 0, d, I);
-    go(k_s1<Real, Dc>, P.s1.n_blocks, 0, d, P.tab, P.s1, (const Real *)x, 0);
+    go(k_s1<Real, Dc, NI>, P.s1.n_blocks, 0, d, tab, sp1, (const Real *)x, 0);
   } else {
-    k_s1<Real, Dc><<<P.s1.n_blocks, NTHR, 0, s>>>(d, P.tab, P.s1, x, 0);
+    k_s1<Real, Dc, NI><<<P.s1.n_blocks, NTHR, 0, s>>>(d, tab, sp1, x, 0);
     e = cudaGetLastError();
   }
   mark(ev, 1, s);
   nvtxRangePop();
   nvtxRangePushA("qg stage 2 (contingencies)");
   if (P.s2.n_blocks > 0) {  // no contingencies: nothing for stage 2
-    if (P.ctg_lazy) go(k_ctg_margin<Real, Dc>, 152 * 4, 0, d, P.tab);
+    if (P.ctg_lazy) go(k_ctg_margin<Real, Dc, NI>, 152 * 4, 0, d, tab);
     const size_t sm2 = ctg_smem_bytes<Real>(P.maxTB, d.score != 0, P.ctg_lazy != 0, P.hot != 0);
-    if (P.ctg_lazy) go(k_s2<Real, Dc, 2>, P.s2.n_blocks, sm2, d, P.tab, P.s2, (const Real *)x, o2);
-    else if (P.ctg_bound) go(k_s2<Real, Dc, 1>, P.s2.n_blocks, sm2, d, P.tab, P.s2, (const Real *)x, o2);
-    else go(k_s2<Real, Dc, 0>, P.s2.n_blocks, sm2, d, P.tab, P.s2, (const Real *)x, o2);
+    if (P.ctg_lazy) go(k_s2<Real, Dc, 2, NI>, P.s2.n_blocks, sm2, d, tab, sp2, (const Real *)x, o2);
+    else if (P.ctg_bound) go(k_s2<Real, Dc, 1, NI>, P.s2.n_blocks, sm2, d, tab, sp2, (const Real *)x, o2);
+    else go(k_s2<Real, Dc, 0, NI>, P.s2.n_blocks, sm2, d, tab, sp2, (const Real *)x, o2);
   }
   mark(ev, 2, s);
   nvtxRangePop();
   nvtxRangePushA("qg stage 3");
-  if (P.tab.s3q > 1) go(k_s3<Real, Dc, S3_SPLIT_MAX>, P.s3.n_blocks, 0, d, P.tab, P.s3, (const Real *)x);
-  else go(k_s3<Real, Dc, 1>, P.s3.n_blocks, 0, d, P.tab, P.s3, (const Real *)x);
+  if (P.tab.s3q > 1) go(k_s3<Real, Dc, S3_SPLIT_MAX, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
+  else go(k_s3<Real, Dc, 1, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
   mark(ev, 3, s);
   nvtxRangePop();
   nvtxRangePushA("qg stage 4");
   // stage 4 with the device updates (small plans on the mixed path) or without them (a separate
   // instantiation: the fused role's registers would cost the lean one its occupancy)
   if (P.tab.fuse) {
-    if (adam) go(k_s4<Real, Dc, true, true>, P.s4.n_blocks, 0, d, P.tab, P.s4, x);
-    else go(k_s4<Real, Dc, false, true>, P.s4.n_blocks, 0, d, P.tab, P.s4, x);
+    if (adam) go(k_s4<Real, Dc, true, true, NI>, P.s4.n_blocks, 0, d, tab, sp4, x);
+    else go(k_s4<Real, Dc, false, true, NI>, P.s4.n_blocks, 0, d, tab, sp4, x);
   } else {
-    if (adam) go(k_s4<Real, Dc, true, false>, P.s4.n_blocks, 0, d, P.tab, P.s4, x);
-    else go(k_s4<Real, Dc, false, false>, P.s4.n_blocks, 0, d, P.tab, P.s4, x);
+    if (adam) go(k_s4<Real, Dc, true, false, NI>, P.s4.n_blocks, 0, d, tab, sp4, x);
+    else go(k_s4<Real, Dc, false, false, NI>, P.s4.n_blocks, 0, d, tab, sp4, x);
   }
   if (P.sp) {
     // sparse mode: adjoint solve eta = Yhat^-1 w at the generator buses, and 1^T eta
@@ -2908,15 +2962,21 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *xv, b
   nvtxRangePop();
   nvtxRangePushA("qg stage 5 + closing kernel");
   if (P.s5.n_blocks > 0) {  // the mixed path's dense mode updates the devices in stage 4
-    if (adam) go(k_s5<Real, Dc, true>, P.s5.n_blocks, 0, d, P.tab, P.s5, x);
-    else go(k_s5<Real, Dc, false>, P.s5.n_blocks, 0, d, P.tab, P.s5, x);
+    if (adam) go(k_s5<Real, Dc, true, NI>, P.s5.n_blocks, 0, d, tab, sp5, x);
+    else go(k_s5<Real, Dc, false, NI>, P.s5.n_blocks, 0, d, tab, sp5, x);
   }
-  if (close) go(k_finish<Real, Dc>, 1, 0, d, P.tab, adam ? 1 : 0);  // the objective, step += 1 with Adam
+  if (close) go(k_finish<Real, Dc, NI>, 1, 0, d, tab, adam ? 1 : 0);  // the objective, step += 1 with Adam
   nvtxRangePop();
   mark(ev, 5, s);
   return e;
 }
 
+template <typename Real, typename Dc>
+cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *x, bool adam, bool close, cudaStream_t s,
+                        cudaEvent_t *ev) {
+  return P.tab.n_inst == 1 ? launch_stages<Real, Dc, 1>(d, P, x, adam, close, s, ev)
+                           : launch_stages<Real, Dc, MAXB>(d, P, x, adam, close, s, ev);
+}
 
 // The contingency kernel's dynamic shared-memory limit is a process-wide function attribute: it is
 // only ever raised, so that creating a handle with smaller blocks never breaks an existing one.
@@ -2928,9 +2988,16 @@ cudaError_t prepare_eval(int maxTB, bool score, bool lazy, bool hot) {
   if (sm > 227 * 1024) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(mu);
   if (sm <= cur) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_s2<Real, Dc, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_s2<Real, Dc, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_s2<Real, Dc, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = cudaSuccess;
+  auto raise = [&](auto kern) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  };
+  raise(k_s2<Real, Dc, 0, 1>);
+  raise(k_s2<Real, Dc, 1, 1>);
+  raise(k_s2<Real, Dc, 2, 1>);
+  raise(k_s2<Real, Dc, 0, MAXB>);
+  raise(k_s2<Real, Dc, 1, MAXB>);
+  raise(k_s2<Real, Dc, 2, MAXB>);
   if (e == cudaSuccess) cur = sm;
   return e;
 }
