@@ -1303,7 +1303,8 @@ bool mixed(const qg_ctx *h) { return h->opt.precision == QG_MIXED; }
 // the objective sum and the step count to a run_finish after the graph's last iteration (fused
 // iterations without a trace); otherwise the evaluation ends with its own closing kernel.
 int run_eval(qg_ctx *h, const void *x, bool adam, double lr, double b1, double b2, double *trace, int trace_len,
-             const double *sched = nullptr, int sched_len = 0, int step_off = 0, bool defer = false) {
+             const double *sched = nullptr, int sched_len = 0, int step_off = 0, bool defer = false,
+             double *obj_out = nullptr, void *g_out = nullptr) {
   cudaEvent_t *ev = h->profiling ? h->ev : nullptr;
   cudaError_t e;
   if (mixed(h)) {
@@ -1311,12 +1312,14 @@ int run_eval(qg_ctx *h, const void *x, bool adam, double lr, double b1, double b
     d.lr = lr; d.b1 = b1; d.b2 = b2; d.aeps = h->opt.adam_eps; d.paper_eps = h->opt.adam_paper_eps;
     d.trace = trace; d.trace_len = trace_len; d.sched = sched; d.sched_len = sched_len;
     d.step_off = step_off;
+    d.obj_out = obj_out; d.g_out = (float *)g_out;
     e = launch_eval<float, df32>(d, h->plan, x, adam, !defer, h->stream, ev);
   } else {
     Dev<double, double> d = h->d64;
     d.lr = lr; d.b1 = b1; d.b2 = b2; d.aeps = h->opt.adam_eps; d.paper_eps = h->opt.adam_paper_eps;
     d.trace = trace; d.trace_len = trace_len; d.sched = sched; d.sched_len = sched_len;
     d.step_off = step_off;
+    d.obj_out = obj_out; d.g_out = (double *)g_out;
     e = launch_eval<double, double>(d, h->plan, x, adam, !defer, h->stream, ev);
   }
   if (e != cudaSuccess) return fail(h, QG_ERR_CUDA, std::string("evaluation launch: ") + cudaGetErrorString(e));
@@ -1412,6 +1415,23 @@ double time_evals(qg_ctx *h, const void *x, int reps, void *flush, size_t flush_
   for (auto &e : ev)
     if (e) cudaEventDestroy(e);
   return ok ? ms / reps : -1.0;
+}
+
+bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+  return a && b && x < y + nb && y < x + na;
+}
+
+// Whether the stage kernels may write the caller's array p (n bytes of elements of size el) while an evaluation
+// reads x (nx bytes): aligned device memory apart from x.
+bool writable(const void *p, size_t n, size_t el, const void *x, size_t nx) {
+  if ((uintptr_t)p % el || overlap(p, n, x, nx)) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice;
 }
 
 // Closing kernel of n deferred iterations: the objective of the last one (read at its schedule
@@ -1746,11 +1766,18 @@ int qg_set_stream(qg_ctx *h, void *stream) {
 int qg_eval_grad(qg_ctx *h, const void *x, double *obj, void *g) {
   NvtxRange range("qg_eval_grad");
   if (!h || !x) return h ? fail(h, QG_ERR_INVALID_ARG, "x is NULL") : QG_ERR_INVALID_ARG;
-  int rc = run_eval(h, x, false, 0, 0, 0, nullptr, 0);
-  if (rc) return rc;
   const size_t rs = mixed(h) ? sizeof(float) : sizeof(double);
-  if (obj) CUDA_TRY(h, cudaMemcpyAsync(obj, h->d_obj, sizeof(double) * h->n_inst, cudaMemcpyDeviceToDevice, h->stream));
-  if (g) CUDA_TRY(h, cudaMemcpyAsync(g, h->d_g, rs * h->n_x, cudaMemcpyDeviceToDevice, h->stream));
+  const size_t ng = rs * h->n_x, no = sizeof(double) * h->n_inst;
+  // the last stages write the caller's arrays along with the handle's (rt617: two copies, 4 us of the 50);
+  // arrays that a kernel must not write that early or cannot take a copy afterwards
+  const bool dg = g && writable(g, ng, rs, x, ng) && !overlap(g, ng, obj, no);
+  const bool dobj = obj && writable(obj, no, sizeof(double), x, ng) && !overlap(g, ng, obj, no);
+  if (dg) bounds_register(g, ng);  // index-checked builds: the caller's arrays
+  if (dobj) bounds_register(obj, no);
+  int rc = run_eval(h, x, false, 0, 0, 0, nullptr, 0, nullptr, 0, 0, false, dobj ? obj : nullptr, dg ? g : nullptr);
+  if (rc) return rc;
+  if (obj && !dobj) CUDA_TRY(h, cudaMemcpyAsync(obj, h->d_obj, no, cudaMemcpyDeviceToDevice, h->stream));
+  if (g && !dg) CUDA_TRY(h, cudaMemcpyAsync(g, h->d_g, ng, cudaMemcpyDeviceToDevice, h->stream));
   return QG_OK;
 }
 

@@ -236,6 +236,8 @@ struct Dev {
   const int *slot_map;                // [n_obj12] stage-1/2 block (launch order) -> slot
   double *obj, *terms;                // [n_inst], [n_inst][N_TERMS]
   Real *g;                            // gradient [n_x]
+  Real *g_out;                        // the caller's arrays written along with g and obj (qg_eval_grad; may be NULL)
+  double *obj_out;
   unsigned int *ticket;               // last-block counter of the stand-alone Adam kernel
   long long *step;                    // Adam step counter (written by closing kernels and that kernel)
   int step_off;                       // iteration k of a graph of several: it reads step + k

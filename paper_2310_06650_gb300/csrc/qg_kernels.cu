@@ -32,6 +32,7 @@
 #include <map>
 #include <mutex>
 #include <cstdint>
+#include <iterator>
 #include <utility>
 #include <vector>
 
@@ -89,9 +90,13 @@ void upload_ranges() {
 void bounds_register(const void *p, size_t bytes) {
   if (!p || !bytes) return;
   std::lock_guard<std::mutex> lock(g_ranges_mu);
-  auto &b = g_ranges[reinterpret_cast<unsigned long long>(p)];
-  if (b == bytes) return;
-  b = bytes;
+  const unsigned long long lo = reinterpret_cast<unsigned long long>(p), hi = lo + bytes;
+  auto known = g_ranges.find(lo);
+  if (known != g_ranges.end() && known->second == bytes) return;
+  // arrays that overlap it are gone: a caller's buffer whose memory has been allocated anew
+  for (auto it = g_ranges.begin(); it != g_ranges.end();)
+    it = it->first < hi && lo < it->first + it->second ? g_ranges.erase(it) : std::next(it);
+  g_ranges[lo] = bytes;
   upload_ranges();
 }
 
@@ -378,6 +383,13 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
   float d;
   asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
+}
+
+// One gradient entry: the handle's copy and, in qg_eval_grad, the caller's (no copy afterwards).
+template <typename Real, typename Dc>
+__device__ __forceinline__ void put_grad(const Dev<Real, Dc> &d, long long k, Real v) {
+  d.g[k] = v;
+  if (d.g_out) d.g_out[k] = v;
 }
 
 struct Where {
@@ -2085,8 +2097,8 @@ __device__ void s4_bus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, Re
           d.av[k2[c]] = s_v[u][c];
         }
       } else {
-        d.g[k2[0]] = gv[u];
-        d.g[k2[1]] = gth[u];
+        put_grad(d, k2[0], gv[u]);
+        put_grad(d, k2[1], gth[u]);
       }
     }
   }
@@ -2139,6 +2151,7 @@ __device__ void final_reduce(const Dev<Real, Dc> &d, const InstTabT<NI> &tab) {
         tot += tv;
       }
       d.obj[b] = tot;
+      if (d.obj_out) d.obj_out[b] = tot;
       if (d.trace) {
         const long long it = *d.step + d.step_off - *d.trace_step0;
         if (it >= 0 && it < d.trace_len) d.trace[it * tab.n_inst + b] = tot;
@@ -2304,10 +2317,10 @@ __device__ void gen_update(const Dev<Real, Dc> &d, const Inst &I, int t, int gl,
       d.av[k4[c]] = vk;
     }
   } else {
-    d.g[g.kp] = gp;
-    d.g[g.kq] = gq;
-    d.g[g.kr] = gr;
-    if (I.uc) d.g[g.ku] = gu;
+    put_grad(d, g.kp, gp);
+    put_grad(d, g.kq, gq);
+    put_grad(d, g.kr, gr);
+    if (I.uc) put_grad(d, g.ku, gu);
   }
 }
 
@@ -2378,7 +2391,7 @@ __device__ void gen_update_lanes(const Dev<Real, Dc> &d, const Inst &I, int t, i
     d.am[k] = mk;
     d.av[k] = vk;
   } else {
-    d.g[k] = grad;
+    put_grad(d, k, grad);
   }
 }
 
@@ -2404,8 +2417,8 @@ __device__ void xf_update(const Dev<Real, Dc> &d, const Inst &I, int t, int xi, 
     adam_update(x[kp], gphi, d.am[kp], d.av[kp], d.lo[kp], d.hi[kp], ac.b1, ac.b2, ac.c1, ac.c2, ac.lr, ac.eps,
                 d.paper_eps);
   } else {
-    d.g[kt] = gtau;
-    d.g[kp] = gphi;
+    put_grad(d, kt, gtau);
+    put_grad(d, kp, gphi);
   }
 }
 
