@@ -787,15 +787,18 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
         I[b].gen_slot0 = gen_slot;
         gen_slot += I[b].gen_nb;
       }
-      add_span(P.s4, per_t, I[b].T, b, R_GBUS);
+      if (bp > SMALL_PLAN) add_span(P.sg, per_t, ceil_div(I[b].T, GB_TC), b, R_GBUS);
+      else add_span(P.s4, per_t, I[b].T, b, R_GBUS);
     }
   else
     add_span(P.s4, ceil_div(H0.n - 1, 32), ceil_div(H0.T, DCF_TC), 0, R_SDCA);
   if (!fuse) {
     // FP64: one warp of pairs per block (GB300's FP64 pipe costs as much for a warp with one active
-    // lane as for a full one), 8 pairs of four lanes each without on-status, else 32 of one
+    // lane as for a full one), 8 pairs of four lanes each without on-status, else 32 of one; whole blocks
+    // where there are several per SM of them (day-ahead grid: 18,000 blocks of one warp took 351 us)
     for (int b = 0; b < B; ++b) {
-      const int gen_pb = h->opt.precision == QG_FP64 ? (I[b].uc ? 32 : 8) : NTHR;
+      const bool big = (long long)I[b].T * I[b].G > 8 * 152 * 64;
+      const int gen_pb = h->opt.precision == QG_FP64 ? (big ? (I[b].uc ? NTHR : NTHR / 4) : I[b].uc ? 32 : 8) : NTHR;
       I[b].gen_first = P.s5.n_blocks;
       I[b].gen_pb = gen_pb;
       I[b].gen_nb = ceil_div((long long)I[b].T * I[b].G, gen_pb);
@@ -1219,6 +1222,7 @@ int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) 
   WR(pf, sTM) WR(qf, sTM) WR(pt, sTM) WR(qt, sTM) WR(qm2, sTM) WR(fre, sTM) WR(fk, sTK) WR(pold, sTG) WR(uold, sTG)
   WR(dP, sTn) WR(dQ, sTn) WR(dZ, sTZ) WR(pm, sPM) WR(pq, sPM) WR(pk, sPK) WR(gF, sTM) WR(avf, sTM) WR(avo, sTM)
   WR(ad, sTM) WR(atx, sTX) WR(pkh, std::max(1LL, hot_elems(P)))
+  if (sizeof(Real) == 8) { WR(sn, sTM) WR(cs, sTM) }
   WD(gip, sGI)
   WF(f32, sTM) WF(fk32, sTK)
 #undef WR
@@ -1580,18 +1584,21 @@ size_t carve_scratch(const qg_ctx *h, unsigned char *base, size_t cap, Dev<Real,
   return off;
 }
 
-// Carve the hot rows' flags and column sums out of [base, base + NOALLOC_HOT_BYTES); false if they do
-// not fit.  They take T M bytes and at most n_mg T Kp elements (Kp < K + 4, n_mg <= M / 64 + 1), and the
-// work buffers hold n_mg T K, 2 ceil(K / 64) T M and more than 12 T M elements: a handle whose work
-// buffers fit 16 MiB fits here.
+// Carve what the 16 MiB limit leaves out of [base, base + NOALLOC_HOT_BYTES): the hot rows' flags and column
+// sums, and the FP64 path's sines and cosines; false if they do not fit.  They take T M bytes, at most n_mg T Kp
+// elements (Kp < K + 4, n_mg <= M / 64 + 1) and 2 T M elements, and the work buffers hold n_mg T K, 2 ceil(K / 64)
+// T M and more than 12 T M elements: a handle whose work buffers fit 16 MiB fits here.
 template <typename Real, typename Dc>
 bool carve_hot(const qg_ctx *h, unsigned char *base, Dev<Real, Dc> &d) {
   const size_t sums = (sizeof(Real) * (size_t)hot_elems(h->plan) + 255) & ~size_t(255);
-  size_t flags = 0;
-  for (int b = 0; b < h->n_inst; ++b) flags += (size_t)h->plan.tab.I[b].T * h->plan.tab.I[b].M;
+  size_t tm = 0;
+  for (int b = 0; b < h->n_inst; ++b) tm += (size_t)h->plan.tab.I[b].T * h->plan.tab.I[b].M;
+  const size_t trig = sizeof(Real) == 8 ? tm : 0;
   d.pkh = (Real *)base;
-  d.hot = base + sums;
-  return sums + flags <= NOALLOC_HOT_BYTES;
+  d.sn = (Real *)(base + sums);
+  d.cs = d.sn + trig;
+  d.hot = (unsigned char *)(d.cs + trig);
+  return sums + 2 * trig * sizeof(Real) + tm <= NOALLOC_HOT_BYTES;
 }
 
 template <typename Real, typename Dc>
@@ -2300,7 +2307,7 @@ int32_t qg_launches_per_eval(const qg_ctx *h) {
   // no contingencies: no stage 2; the on-demand contingency path adds the clearance kernel before it
   const int s2 = P.s2.n_blocks > 0 ? 1 + (P.ctg_lazy ? 1 : 0) : 0;
   // + 1: the closing kernel (the mixed path's dense mode updates the devices in stage 4)
-  if (!P.sp) return 3 + s2 + (P.s5.n_blocks > 0 ? 1 : 0) + 1;
+  if (!P.sp) return 3 + s2 + (P.sg.n_blocks > 0 ? 1 : 0) + (P.s5.n_blocks > 0 ? 1 : 0) + 1;
   return 4 + s2 + 3 + (P.sp_tail ? 6 : 0) + (P.sp_bw_blocks > 0 ? 1 : 0) + (P.sp_bwa_blocks > 0 ? 1 : 0) + 1;
 }
 

@@ -32,6 +32,7 @@ constexpr int DCF_BM = 32, DCF_TC = 8; // forward DC tile: 32 branches x 8 perio
 constexpr int PACK = 32;               // CSR entries per warp pack (rows never straddle packs)
 constexpr int PACKS_PER_BLOCK = NTHR / 32;
 constexpr int S4_PACKS = 2;            // branch-end CSR packs per warp in the bus gather of stage 4, at most
+constexpr int GB_TC = 4;               // periods per warp of k_gbus
 constexpr int S3_SPLIT_MAX = 4;        // threads per branch-period in stage 3 (InstTab::s3q), at most
 
 // One instance of a batch.  Entity ids inside the kernels are global (offset by
@@ -207,6 +208,7 @@ struct Dev {
   int lodf_dtype;
   // work buffers
   Real *pf, *qf, *pt, *qt, *qm2;      // [sum T M]
+  Real *sn, *cs;                      // [sum T M] FP64 path only: sine and cosine of the angle across the branch
   unsigned char *qside;               // [sum T M] 1 if the "to" end carries the larger |q|
   Real *fre;                          // [sum T M] base DC flows
   float *f32;                         // [sum T M] FP32 copy (FP64 path screening)
@@ -254,6 +256,7 @@ struct Dev {
 
 struct Plan {
   Spans s1, s2, s3, s4, s5;
+  Spans sg;   // adjoint DC products of large dense plans (k_gbus; otherwise stage 4's R_GBUS)
   InstTab tab;
   long long n_x;
   int maxT;

@@ -478,7 +478,7 @@ constexpr int GBC = 128;  // generator-bus chunk of the DC products
 // with 1 - cos d = sin^2 d / (1 + cos d) while cos d > 0.
 template <typename Real, typename Dc>
 __device__ __forceinline__ void pi_flow(const Dev<Real, Dc> &d, const Inst &I, int t, int jg, const Real *__restrict__ x,
-                                        Real &pf, Real &qf, Real &pt, Real &qt) {
+                                        Real &pf, Real &qf, Real &pt, Real &qt, Real &sn, Real &cs) {
   const int2 ft = d.br_end[jg];
   const Real *v = x + I.x0 + (long long)t * I.n;
   const Real *th = v + (long long)I.T * I.n;
@@ -488,7 +488,6 @@ __device__ __forceinline__ void pi_flow(const Dev<Real, Dc> &d, const Inst &I, i
   const Real vf = v[ft.x] / tau, vo = v[ft.y];
   const Real dl = th[ft.x] - th[ft.y] - phi;
   const Real g = d.br_g[jg], bb = d.br_b[jg], hch = d.br_hch[jg];
-  Real sn, cs;
   dsincos(dl, &sn, &cs);
   const Real vv = vf * vo;
   const Real dv = vf - vo;
@@ -507,9 +506,13 @@ __device__ void s1_branch(const Dev<Real, Dc> &d, const Inst &I, int t, int sub,
   const int jg = I.br0 + j;
   const Real smax = d.br_smax[jg];
   const Real wt = d.dt[I.tp0 + t] * d.c_s * hp.beta;  // loaded before the stores below
-  Real pf, qf, pt, qt;
-  pi_flow(d, I, t, jg, x, pf, qf, pt, qt);
+  Real pf, qf, pt, qt, sn, cs;
+  pi_flow(d, I, t, jg, x, pf, qf, pt, qt, sn, cs);
   const long long e = I.tm0 + (long long)t * I.M + j;
+  if constexpr (sizeof(Real) == 8) {  // stage 3 takes them from here: a sincos is a long FP64 sequence
+    d.sn[e] = sn;
+    d.cs[e] = cs;
+  }
   d.pf[e] = pf;
   d.qf[e] = qf;
   d.pt[e] = pt;
@@ -738,8 +741,8 @@ __device__ void s1_bus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, co
   const long long ti = I.tb0 + (long long)t * I.n + (row >= 0 ? row : 0);
   Real P = 0, Q = 0;
   if (kind <= 1) {
-    Real pf, qf, pt, qt;
-    pi_flow(d, I, t, I.br0 + id, x, pf, qf, pt, qt);
+    Real pf, qf, pt, qt, sn, cs;
+    pi_flow(d, I, t, I.br0 + id, x, pf, qf, pt, qt, sn, cs);
     P = kind == 0 ? pf : pt;
     Q = kind == 0 ? qf : qt;
   } else if (kind == 2) {  // a producer supplies (-), a consumer draws (+)
@@ -1803,7 +1806,7 @@ __device__ void fold_slots(const Dev<Real, Dc> &d, const Inst &I, int r) {
   }
 }
 
-template <typename Real, typename Dc, int SPLIT, int NI>
+template <typename Real, typename Dc, int SPLIT, bool HOT, int NI>
 __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __grid_constant__ Dev<Real, Dc> d,
                                              const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              const Real *__restrict__ x) {
@@ -1837,8 +1840,12 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
   const long long tb = I.tb0 + (long long)t * I.n;
   Real gpf = 0, gpt = 0, gqf = 0, gqt = 0, pf = 0, qf = 0, pt = 0, qt = 0, vf0 = 1, vo = 1, thf = 0, tho = 0;
   bool qto = false;
-  Real tau = Real(1), phi = Real(0);
+  Real tau = Real(1), phi = Real(0), sn = 0, cs = 1;
   if (lead) {
+    if constexpr (sizeof(Real) == 8) {
+      sn = d.sn[e];
+      cs = d.cs[e];
+    }
     gpf = d.dP[tb + ft.x];
     gpt = d.dP[tb + ft.y];
     gqf = d.dQ[tb + ft.x];
@@ -1859,11 +1866,11 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       phi = x[I.xtau0 + (long long)(I.T + t) * I.X + xi0];
     }
   }
-  Real gF = 0, gq2 = 0, gk = 0, gh = 0, zk = 0;  // gh: the hot rows' share of gk
+  Real gF = 0, gq2 = 0, gk = 0, zk = 0;
   // row partials of the outage tiles whose 64-row tile had an overload (flagged by stage 2), or, for a hot
   // row, of the first outage tile of each of s2_hot's chunks: few tiles are read unconditionally and
   // selected (no dependent load); of many, the set ones are summed in order
-  const bool hot = on && I.hot && d.hot[e] != 0;
+  const bool hot = HOT && on && I.hot && d.hot[e] != 0;
   if (I.n_kt > 16 * SPLIT) {
     for (int k0 = 0; k0 < I.n_kt; k0 += 32) {
       unsigned set = 0;
@@ -1899,19 +1906,17 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       }
     }
     if (kx >= 0) {
-      if (SPLIT > 1 || !I.hot) {
+      if (!HOT || !I.hot) {
 #pragma unroll 8
         for (int mg = q; mg < I.n_mg; mg += SPLIT) gk += d.pk[I.pk0 + ((long long)mg * I.T + t) * I.K + kx];
-#pragma unroll 8
-        for (int mg = q; mg < I.hot; mg += SPLIT) gh += d.pkh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + kx];
       }
       if (d.score) {
         for (int mg = q; mg < I.n_mg; mg += SPLIT) zk += d.pz[I.pk0 + ((long long)mg * I.T + t) * I.K + kx];
-        for (int mg = q; mg < I.hot; mg += SPLIT) zk += d.pzh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + kx];
+        for (int mg = q; HOT && mg < I.hot; mg += SPLIT) zk += d.pzh[I.ph0 + ((long long)mg * I.T + t) * I.Kp + kx];
       }
     }
   }
-  if (SPLIT == 1 && I.hot) {
+  if (HOT && I.hot) {
     // many column partials (large plans, where few branches are outages): the whole warp sums those of
     // each of its outage branches, a lane every 32nd, instead of one lane walking them all
     const int lane = threadIdx.x & 31;
@@ -1927,7 +1932,6 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
       if (lane == src) gk = s;
     }
   }
-  gk += gh;
 #pragma unroll
   for (int o = 1; o < SPLIT; o <<= 1) {
     gF += __shfl_xor_sync(0xffffffffu, gF, o);
@@ -1959,8 +1963,7 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
     else gqf += Real(2) * qf * gq2;
     const int xi = xi0;
     const Real vf = vf0 / tau;  // vf stands for v_f / tau
-    Real sn, cs;
-    dsincos(thf - tho - phi, &sn, &cs);
+    if constexpr (sizeof(Real) == 4) dsincos(thf - tho - phi, &sn, &cs);
     const Real bc = bb + hch;
     const Real vv = vf * vo;
     const Real A = -g * cs - bb * sn, B = bb * cs - g * sn, C = -g * cs + bb * sn, D = bb * cs + g * sn;
@@ -2468,7 +2471,7 @@ __global__ void __launch_bounds__(NTHR) k_s5(const __grid_constant__ Dev<Real, D
       const Dc *et = d.gip + I.gi0 + (long long)tg * (I.Gc + 1);  // written by stage 4 or the adjoint solve
       eta = d.sp ? DcOps<Dc>::add(et[g.gb], DcOps<Dc>::neg(DcOps<Dc>::mul(et[I.Gc], DcOps<Dc>::inv_n(I)))) : et[g.gb];
     }
-    if (threadIdx.x < 32) gen_update_lanes<Real, Dc, ADAM>(d, I, tg, gl, part, on, g, eta, ac, acc, x);
+    if ((int)(threadIdx.x & ~31) < 4 * I.gen_pb) gen_update_lanes<Real, Dc, ADAM>(d, I, tg, gl, part, on, g, eta, ac, acc, x);
     write_obj(d.objp, d.n_obj12 + I.gen_slot0 + (blockIdx.x - I.gen_first), acc);
   } else {
     Obj3<Dc> acc = obj3<Dc>(T_COST, T_ZHEAD, T_ZRAMP);
@@ -2528,7 +2531,75 @@ __device__ void s4_sdca(const Dev<Real, Dc> &d, const Inst &I, int tc, int sub) 
 // stored for stage 5, which updates 32 (FP64 path) or 256 devices per block: the FP64 pipe takes
 // about as long for a warp with one active lane as for a full one, and large plans would get one
 // objective slot per stage-4 block.
-template <typename Real, typename Dc, bool ADAM, bool FUSE>
+// Products of a column A (of I.M branches) with nt <= NT periods of dz/df, one warp: lanes stride over the
+// branches, four accumulators per period, a fixed-order shuffle reduction (each period's sum has the same order
+// whatever NT is); the sums are valid in lane 0.
+template <int NT, typename Real, typename Dc>
+__device__ __forceinline__ void gbus_products(const Inst &I, const Dc *__restrict__ A, const Real *__restrict__ gf, int nt,
+                                              Dc *eta) {
+  constexpr int UN = NT == 1 ? 8 : 4;  // strides whose loads are issued together
+  const int lane = threadIdx.x & 31;
+  Dc a[NT][4];
+#pragma unroll
+  for (int i = 0; i < NT; ++i)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[i][k] = DcOps<Dc>::zero();
+  for (int m0 = 0; m0 < I.M; m0 += UN * 32) {
+    Dc av[UN];
+    Real gv[NT][UN];
+#pragma unroll
+    for (int k = 0; k < UN; ++k) {
+      const int m = m0 + k * 32 + lane;
+      av[k] = m < I.M ? A[m] : DcOps<Dc>::zero();
+#pragma unroll
+      for (int i = 0; i < NT; ++i) gv[i][k] = m < I.M && i < nt ? gf[(long long)i * I.M + m] : Real(0);
+    }
+#pragma unroll
+    for (int i = 0; i < NT; ++i)
+#pragma unroll
+      for (int k = 0; k < UN; ++k) DcOps<Dc>::mac(a[i][k & 3], av[k], DcOps<Dc>::from_real(gv[i][k]));
+  }
+#pragma unroll
+  for (int i = 0; i < NT; ++i) {
+    eta[i] = DcOps<Dc>::add(DcOps<Dc>::add(a[i][0], a[i][1]), DcOps<Dc>::add(a[i][2], a[i][3]));
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) eta[i] = DcOps<Dc>::add(eta[i], DcOps<Dc>::shfl_down(eta[i], k));
+  }
+}
+
+// The products of one column with nt <= NT periods from t0 on, alone (plans whose stage 5 updates the devices).
+template <int NT, typename Real, typename Dc>
+__device__ __forceinline__ void gbus_column(const Dev<Real, Dc> &d, const Inst &I, int t0, int nt, int c) {
+  const int lane = threadIdx.x & 31;
+  const Dc *A = d.ptdfaT + I.pg0 + (long long)(c < I.Gc ? c : 0) * I.M;
+  if (c < I.Gc)  // the column is static: start bringing its lines to L2 before the wait
+    for (long long off = (long long)lane * 128; off < (long long)I.M * (long long)sizeof(Dc); off += 32 * 128)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(A) + off));
+  pdl_wait();
+  if (c >= I.Gc) return;  // whole warp
+  Dc eta[NT];
+  gbus_products<NT>(I, A, d.gF + I.tm0 + (long long)t0 * I.M, nt, eta);
+  if (lane == 0)
+#pragma unroll
+    for (int i = 0; i < NT; ++i)
+      if (i < nt) d.gip[I.gi0 + (long long)(t0 + i) * (I.Gc + 1) + c] = eta[i];
+}
+
+// Adjoint DC products of large dense plans: a warp takes its column with GB_TC periods at a time, so that the
+// column (the static bulk of the traffic) comes from L2 once per GB_TC periods and the block's warps share the
+// rows of dz/df in L1 (1,576 buses, 48 periods: stage 4 48 us with one period per warp, of which 300 MB of
+// L2 reads).  A kernel of its own: its registers would cost stage 4's bus gather its occupancy (batch of 32:
+// 251 -> 275 us).
+template <typename Real, typename Dc, int NI>
+__global__ void __launch_bounds__(NTHR) k_gbus(const __grid_constant__ Dev<Real, Dc> d,
+                                               const __grid_constant__ InstTabT<NI> tab,
+                                               const __grid_constant__ SpansT<NI> S) {
+  const Where w = locate(S);
+  const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
+  gbus_column<GB_TC>(d, I, w.t * GB_TC, min(GB_TC, I.T - w.t * GB_TC), w.sub * (NTHR / 32) + (threadIdx.x >> 5));
+}
+
+template <typename Real, typename Dc, bool ADAM>
 __device__ void s4_gbus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, const AdamCoef<Real> &ac,
                         Obj3<Dc> &acc, Real *__restrict__ x) {
   const int lane = threadIdx.x & 31;
@@ -2536,7 +2607,7 @@ __device__ void s4_gbus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, c
   const bool col = c < I.Gc;
   // data no earlier stage writes: the bus's first 32 devices (more take further rounds after the wait)
   int q0 = 0, q1 = 0;
-  if (FUSE && col && c < I.Gb) {
+  if (col && c < I.Gb) {
     q0 = d.gb_ptr[I.gb0 + c];
     q1 = d.gb_ptr[I.gb0 + c + 1];
   }
@@ -2550,26 +2621,8 @@ __device__ void s4_gbus(const Dev<Real, Dc> &d, const Inst &I, int t, int sub, c
   pdl_wait();
   if (!col) return;  // whole warp
   const Real *gf = d.gF + I.tm0 + (long long)t * I.M;
-  Dc a[4] = {DcOps<Dc>::zero(), DcOps<Dc>::zero(), DcOps<Dc>::zero(), DcOps<Dc>::zero()};
-  for (int m0 = 0; m0 < I.M; m0 += 8 * 32) {  // 8 strides per batch: their loads are issued together
-    Dc av[8];
-    Real gv[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int m = m0 + k * 32 + lane;
-      av[k] = m < I.M ? A[m] : DcOps<Dc>::zero();
-      gv[k] = m < I.M ? gf[m] : Real(0);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) DcOps<Dc>::mac(a[k & 3], av[k], DcOps<Dc>::from_real(gv[k]));
-  }
-  Dc eta = DcOps<Dc>::add(DcOps<Dc>::add(a[0], a[1]), DcOps<Dc>::add(a[2], a[3]));
-#pragma unroll
-  for (int k = 16; k > 0; k >>= 1) eta = DcOps<Dc>::add(eta, DcOps<Dc>::shfl_down(eta, k));
-  if (!FUSE) {
-    if (lane == 0) d.gip[I.gi0 + (long long)t * (I.Gc + 1) + c] = eta;
-    return;
-  }
+  Dc eta;
+  gbus_products<1>(I, A, gf, 1, &eta);
   eta = DcOps<Dc>::bcast(eta);
   if (c >= I.Gb) {
     if (lane == 0) xf_update<Real, Dc, ADAM>(d, I, t, c - I.Gb, DcOps<Dc>::to_real(eta), x, ac);
@@ -2608,9 +2661,13 @@ __global__ void __launch_bounds__(NTHR) k_s4(const __grid_constant__ Dev<Real, D
   } else if (w.role == R_SDCA) {
     s4_sdca(d, I, w.t, w.sub);
   } else {  // R_GBUS
-    Obj3<Dc> acc = obj3<Dc>(T_COST, T_ZHEAD, T_ZRAMP);
-    s4_gbus<Real, Dc, ADAM, FUSE>(d, I, w.t, w.sub, ac, acc, x);
-    if (FUSE) write_obj(d.objp, d.n_obj12 + I.gen_slot0 + (blockIdx.x - I.gen_first), acc);
+    if constexpr (FUSE) {
+      Obj3<Dc> acc = obj3<Dc>(T_COST, T_ZHEAD, T_ZRAMP);
+      s4_gbus<Real, Dc, ADAM>(d, I, w.t, w.sub, ac, acc, x);
+      write_obj(d.objp, d.n_obj12 + I.gen_slot0 + (blockIdx.x - I.gen_first), acc);
+    } else {
+      gbus_column<1>(d, I, w.t, 1, w.sub * (NTHR / 32) + (threadIdx.x >> 5));
+    }
   }
 }
 
@@ -2898,7 +2955,7 @@ static cudaError_t launch_stages(const Dev<Real, Dc> &d, const Plan &P, const vo
                                  cudaStream_t s, cudaEvent_t *ev) {
   const InstTabT<NI> tab = table<NI>(P.tab);
   const SpansT<NI> sp1 = spans<NI>(P.s1), sp2 = spans<NI>(P.s2), sp3 = spans<NI>(P.s3), sp4 = spans<NI>(P.s4),
-                   sp5 = spans<NI>(P.s5);
+                   sp5 = spans<NI>(P.s5), spg = spans<NI>(P.sg);
   Real *x = const_cast<Real *>(static_cast<const Real *>(xv));
   const int o2 = P.s1.n_blocks;
   // with timing events between the kernels, launch them plainly so each event brackets one kernel
@@ -2950,11 +3007,13 @@ static cudaError_t launch_stages(const Dev<Real, Dc> &d, const Plan &P, const vo
   mark(ev, 2, s);
   nvtxRangePop();
   nvtxRangePushA("qg stage 3");
-  if (P.tab.s3q > 1) go(k_s3<Real, Dc, S3_SPLIT_MAX, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
-  else go(k_s3<Real, Dc, 1, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
+  if (P.tab.s3q > 1) go(k_s3<Real, Dc, S3_SPLIT_MAX, false, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
+  else if (P.hot) go(k_s3<Real, Dc, 1, true, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
+  else go(k_s3<Real, Dc, 1, false, NI>, P.s3.n_blocks, 0, d, tab, sp3, (const Real *)x);
   mark(ev, 3, s);
   nvtxRangePop();
   nvtxRangePushA("qg stage 4");
+  if (P.sg.n_blocks > 0) go(k_gbus<Real, Dc, NI>, P.sg.n_blocks, 0, d, tab, spg);
   // stage 4 with the device updates (small plans on the mixed path) or without them (a separate
   // instantiation: the fused role's registers would cost the lean one its occupancy)
   if (P.tab.fuse) {
