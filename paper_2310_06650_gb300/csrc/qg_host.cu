@@ -650,7 +650,7 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
   // at an iterate without overloads 113 -> 118 us, with 10 hot rows per period 180 -> 157; mixed, stage 2
   // 16.2 us in the screen, 15.5-20 us with.
   const bool hot_rows = (el_all > 0 && 2 * el_large >= el_all) || (h->opt.precision == QG_FP64 && bp > SMALL_PLAN);
-  P.tab.s3q = small_mixed ? S3_SPLIT_MAX : 1;
+  P.tab.s3q = small_mixed && !hot_rows ? S3_SPLIT_MAX : 1;  // (a hot plan of few periods has many partials to sum)
   int bus0 = 0, br0 = 0, gen0 = 0, zone0 = 0, ctg0 = 0, gb0 = 0, tp0 = 0, bal0 = 0, adj0 = 0;
   for (int b = 0; b < B; ++b) {
     const HostInst &H = h->hi[b];
