@@ -794,11 +794,11 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
     add_span(P.s4, ceil_div(H0.n - 1, 32), ceil_div(H0.T, DCF_TC), 0, R_SDCA);
   if (!fuse) {
     // FP64: one warp of pairs per block (GB300's FP64 pipe costs as much for a warp with one active
-    // lane as for a full one), 8 pairs of four lanes each without on-status, else 32 of one; whole blocks
+    // lane as for a full one), 8 pairs of four lanes each; whole blocks
     // where there are several per SM of them (day-ahead grid: 18,000 blocks of one warp took 351 us)
     for (int b = 0; b < B; ++b) {
       const bool big = (long long)I[b].T * I[b].G > 8 * 152 * 64;
-      const int gen_pb = h->opt.precision == QG_FP64 ? (big ? (I[b].uc ? NTHR : NTHR / 4) : I[b].uc ? 32 : 8) : NTHR;
+      const int gen_pb = h->opt.precision == QG_FP64 ? (big ? NTHR / 4 : 8) : NTHR;
       I[b].gen_first = P.s5.n_blocks;
       I[b].gen_pb = gen_pb;
       I[b].gen_nb = ceil_div((long long)I[b].T * I[b].G, gen_pb);

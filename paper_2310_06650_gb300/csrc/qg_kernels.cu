@@ -2327,13 +2327,14 @@ __device__ void gen_update(const Dev<Real, Dc> &d, const Inst &I, int t, int gl,
   }
 }
 
-// The FP64 path's device update without on-status variables, one (period, device) pair over four
-// lanes (part = lane & 3): 0 the energy cost, eta, the balance adjoint, the headroom and the ramp
-// into period t, and p's update; 1 q's; 2 r's (with the headroom derivative from lane 0); 3 the
-// ramp terms of period t + 1 that involve p_t (handed to lane 0).  Each gradient is summed in the
-// order of gen_update, so the results are bitwise its; the dependent FP64 chain (square roots and
-// divisions of the soft-ReLUs and of Adam) is about a third as long, and the work spreads over
-// four times as many warps.  Every lane of the warp calls it (the shuffles are warp-wide).
+// The FP64 path's device update, one (period, device) pair over four lanes (part = lane & 3): 0 the energy cost,
+// eta, the balance adjoint, the headroom and the ramp into period t, and p's update; 1 q's (with its u-scaled
+// limits); 2 r's (with the headroom derivative from lane 0) and the limit p >= pmin u (handed to lane 0); 3 the
+// ramp terms of period t + 1 that involve p_t (handed to lane 0) and, with on-status, its costs and u's update
+// (the limits' derivatives from the other lanes).  The dependent FP64 chain (square roots and divisions of the
+// soft-ReLUs and of Adam) is about a third as long as one lane's, and the work spreads over four times as many
+// warps.  Without on-status variables each gradient is summed in the order of gen_update.  Every lane of the
+// warp calls it (the shuffles are warp-wide).
 template <typename Real, typename Dc, bool ADAM>
 __device__ void gen_update_lanes(const Dev<Real, Dc> &d, const Inst &I, int t, int gl, int part, bool on,
                                  const GenIn<Real> &g, Dc eta, const AdamCoef<Real> &ac, Obj3<Dc> &acc,
@@ -2341,7 +2342,7 @@ __device__ void gen_update_lanes(const Dev<Real, Dc> &d, const Inst &I, int t, i
   const long long G = I.G;
   const HP<Real> hp = hparams(d);
   const Real wr = d.rho * hp.beta;
-  Real grad = 0, hd = 0, rp = 0;
+  Real grad = 0, hd = 0, rp = 0, lo_p = 0, lim_u = 0;  // hd, rp, lo_p, lim_u: handed to other lanes of the pair
   if (on) {
     const Real dt = d.dt[I.tp0 + t];
     const long long tb = I.tb0 + (long long)t * I.n;
@@ -2352,7 +2353,7 @@ __device__ void gen_update_lanes(const Dev<Real, Dc> &d, const Inst &I, int t, i
       energy_cost(d, g, en, den);
       grad = dt * g.sg * den + g.sg * (DcOps<Dc>::to_real(eta) - d.dP[tb + g.bus]);
       acc.v[0] = DcOps<Dc>::from_real(dt * (g.sg * en + g.cr * g.r));
-      soft_relu(Real(p64 + (double)g.r - g.pmax64), hp.eps, val, der);
+      soft_relu(Real(p64 + (double)g.r - g.pmax64 * (double)g.u), hp.eps, val, der);  // u = 1 without on-status
       acc.v[1] = DcOps<Dc>::from_real(wr * val);
       hd = wr * der;
       grad += hd;
@@ -2367,28 +2368,68 @@ __device__ void gen_update_lanes(const Dev<Real, Dc> &d, const Inst &I, int t, i
       }
     } else if (part == 1) {
       grad = -g.sg * d.dQ[tb + g.bus];
+      if (I.uc) {  // qmin u <= q <= qmax u
+        const int gg = I.gen0 + gl;
+        Real v1, d1, v2, d2;
+        soft_relu(Real((double)g.q - d.lim_qmax[gg] * (double)g.u), hp.eps, v1, d1);
+        soft_relu(Real(d.lim_qmin[gg] * (double)g.u - (double)g.q), hp.eps, v2, d2);
+        acc.v[1] = DcOps<Dc>::from_real(wr * (v1 + v2));
+        grad += wr * (d1 - d2);
+        lim_u = wr * (d.gen_qmin[gg] * d2 - d.gen_qmax[gg] * d1);
+      }
     } else if (part == 2) {
       grad = dt * g.cr - d.dZ[I.tz0 + (long long)t * I.Z + g.zn];
-    } else if (t + 1 < I.T) {  // ramp terms of period t + 1 that involve p_t
-      const double pn = ADAM ? d.pold[ko + G] : x[g.kp + G];
-      const double lim = g.ramp64 * d.lim_dt[I.tp0 + t + 1];
-      Real v1, d1, v2, d2;
-      soft_relu(Real(pn - p64 - lim), hp.eps, v1, d1);
-      soft_relu(Real(p64 - pn - lim), hp.eps, v2, d2);
-      rp = wr * (d2 - d1);
+      if (I.uc) {  // p >= pmin u
+        const int gg = I.gen0 + gl;
+        Real v1, d1;
+        soft_relu(Real(d.lim_pmin[gg] * (double)g.u - p64), hp.eps, v1, d1);
+        acc.v[1] = DcOps<Dc>::from_real(wr * v1);
+        lo_p = wr * d1;
+        lim_u = d.gen_pmin[gg] * lo_p;
+      }
+    } else {
+      if (I.uc) {  // on cost, startup max(u_t - u_{t-1}, 0) and shutdown max(u_{t-1} - u_t, 0) (Example 2)
+        const int gg = I.gen0 + gl;
+        const Real csu = d.gen_csu[gg], csd = d.gen_csd[gg], con = d.gen_con[gg];
+        const Real up = t >= 1 ? (ADAM ? d.uold[ko - G] : x[g.ku - G]) : d.gen_uinit[gg];
+        const Real du = g.u - up;
+        acc.v[0] = DcOps<Dc>::from_real(dt * con * g.u + csu * fmax(du, Real(0)) + csd * fmax(-du, Real(0)));
+        grad = dt * con + (du > Real(0) ? csu : Real(0)) - (du < Real(0) ? csd : Real(0));
+        if (t + 1 < I.T) {
+          const Real dn = (ADAM ? d.uold[ko + G] : x[g.ku + G]) - g.u;
+          grad -= (dn > Real(0) ? csu : Real(0)) - (dn < Real(0) ? csd : Real(0));
+        }
+      }
+      if (t + 1 < I.T) {  // ramp terms of period t + 1 that involve p_t
+        const double pn = ADAM ? d.pold[ko + G] : x[g.kp + G];
+        const double lim = g.ramp64 * d.lim_dt[I.tp0 + t + 1];
+        Real v1, d1, v2, d2;
+        soft_relu(Real(pn - p64 - lim), hp.eps, v1, d1);
+        soft_relu(Real(p64 - pn - lim), hp.eps, v2, d2);
+        rp = wr * (d2 - d1);
+      }
     }
   }
   const Real from3 = __shfl_xor_sync(0xffffffffu, rp, 3);  // lane 3 -> lane 0 of the pair
   const Real from0 = __shfl_xor_sync(0xffffffffu, hd, 2);  // lane 0 -> lane 2 of the pair
-  if (!on || part == 3) return;
+  if (I.uc) {  // uniform: every lane of the warp
+    const Real low = __shfl_xor_sync(0xffffffffu, lo_p, 2);   // lane 2 -> lane 0
+    const Real lu1 = __shfl_xor_sync(0xffffffffu, lim_u, 2);  // lane 1 -> lane 3
+    const Real lu2 = __shfl_xor_sync(0xffffffffu, lim_u, 1);  // lane 2 -> lane 3
+    const Real h3 = __shfl_xor_sync(0xffffffffu, hd, 3);      // lane 0 -> lane 3
+    if (part == 0) grad -= low;
+    if (part == 3) grad += lu1 + lu2 - g.pmax * h3;
+  }
+  if (!on || (part == 3 && !I.uc)) return;
   if (part == 0 && t + 1 < I.T) grad += from3;
   if (part == 2) grad += from0;
-  const long long k = part == 0 ? g.kp : part == 1 ? g.kq : g.kr;
+  const long long k = part == 0 ? g.kp : part == 1 ? g.kq : part == 2 ? g.kr : g.ku;
   if (ADAM) {
-    Real xk = part == 0 ? g.p : part == 1 ? g.q : g.r;
+    Real xk = part == 0 ? g.p : part == 1 ? g.q : part == 2 ? g.r : g.u;
     Real mk = g.am[0], vk = g.av[0], lo = g.lo[0], hi = g.hi[0];
     if (part == 1) { mk = g.am[1]; vk = g.av[1]; lo = g.lo[1]; hi = g.hi[1]; }
     if (part == 2) { mk = g.am[2]; vk = g.av[2]; lo = g.lo[2]; hi = g.hi[2]; }
+    if (part == 3) { mk = g.am[3]; vk = g.av[3]; lo = g.lo[3]; hi = g.hi[3]; }
     adam_update(xk, grad, mk, vk, lo, hi, ac.b1, ac.b2, ac.c1, ac.c2, ac.lr, ac.eps, d.paper_eps);
     x[k] = xk;
     d.am[k] = mk;
@@ -2459,7 +2500,7 @@ __global__ void __launch_bounds__(NTHR) k_s5(const __grid_constant__ Dev<Real, D
   if (w.role == R_XF) {
     pdl_wait();
     s5_xf<Real, Dc, ADAM>(d, I, t, w.sub, x, ac);
-  } else if (sizeof(Real) == 8 && !I.uc) {  // FP64 without on-status: four lanes per pair
+  } else if (sizeof(Real) == 8) {  // FP64: four lanes per pair
     Obj3<Dc> acc = obj3<Dc>(T_COST, T_ZHEAD, T_ZRAMP);
     const int e = w.sub * I.gen_pb + (int)(threadIdx.x >> 2), part = threadIdx.x & 3;
     const bool on = (int)threadIdx.x < 4 * I.gen_pb && e < I.T * I.G;
