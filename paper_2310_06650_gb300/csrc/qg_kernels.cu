@@ -1326,41 +1326,59 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
           if (lane == 0) s_cand[cpar] = 1;
           const Real w = __ldg(d.dt + I.tp0 + t0 + tl) * d.c_s * hp.beta;
           Real gm[4] = {0, 0, 0, 0}, gq[4] = {0, 0, 0, 0}, gk[4] = {0, 0, 0, 0}, zc[4] = {0, 0, 0, 0};
-          if (F64 ? mx >= 0.f : mx > 0.f) {
+          if constexpr (F64) {
+            // each lane walks its own candidates: as many rounds as the lane with the most has, where a walk over
+            // the 16 elements took a round (some 30 instructions of the FP64 pipe) per element that any lane had
+            // (150-bus grid, stage 2: 18.3 -> 15.7 us)
+            unsigned cm = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) cm |= y[i][j] >= 0.f ? 1u << (4 * i + j) : 0u;  // NaN (pad, outaged branch) fails
+            for (; cm; cm &= cm - 1) {
+              const int e = __ffs(cm) - 1, ei = e >> 2, ej = e & 3, mm = rq * 4 + ei;
+              const Real q2 = d.qm2[I.tm0 + (long long)(t0 + tl) * I.M + m0 + mm];
+              const Real Lx = (Real)d.lodf64[I.l0 + (long long)(m0 + mm) * I.Kp + kc + ej];
+              const Real Fx = s_f64m[tl * CT_BM + mm] + Lx * s_f64k[tl * CT_BK + cq * 4 + ej];
+              const Real a2 = Fx * Fx + q2;
+              if (a2 - s_s2[mm] <= Real(0)) continue;
+              Real val, dd;
+              ctg_element(a2, s_s2[CT_BM + mm], eps, w, val, dd);
+              const Real z = w * (val - eps), dF = dd * Fx, dk = dF * Lx;
+              const Real dq = Real(0.5) * dd;  // dz/dqmax2 = w sigma' / (2 s)
+              obj += z;
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                gm[q] += q == ei ? dF : Real(0);
+                gq[q] += q == ei ? dq : Real(0);
+                gk[q] += q == ej ? dk : Real(0);
+                if (score) zc[q] += q == ej ? z : Real(0);
+              }
+            }
+          } else if (mx > 0.f) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const int mm = rq * 4 + i;
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                if (!(F64 ? y[i][j] >= 0.f : y[i][j] > 0.f)) continue;  // NaN (pad, outaged branch) fails too
+                if (!(y[i][j] > 0.f)) continue;  // NaN (pad, outaged branch) fails too
                 const Real q2 = d.qm2[I.tm0 + (long long)(t0 + tl) * I.M + m0 + mm];
                 Real Fx, Lx, dd;
-                if (F64) {
-                  Lx = (Real)d.lodf64[I.l0 + (long long)(m0 + mm) * I.Kp + kc + j];
-                  Fx = s_f64m[tl * CT_BM + mm] + Lx * s_f64k[tl * CT_BK + cq * 4 + j];
-                  const Real a2 = Fx * Fx + q2;
-                  if (a2 - s_s2[mm] <= Real(0)) continue;
-                  Real val;
-                  ctg_element(a2, s_s2[CT_BM + mm], eps, w, val, dd);
-                  obj += w * (val - eps);
-                  zc[j] += w * (val - eps);
-                } else {
-                  // mixed path: s = sqrt(F^2 + qmax2) and the soft-ReLU through reciprocal square
-                  // roots (a few units in the last place, below the FP32 error of F itself)
-                  float l0, l1;
-                  unpack2(Lp[i >> 1][j], l0, l1);
-                  Lx = (i & 1) ? l1 : l0;
-                  Fx = F[i][j];
-                  const float a2 = __fmaf_rn(F[i][j], F[i][j], (float)q2);
-                  const float ra = rsqrtf(a2);
-                  const float u = fmaxf(__fmaf_rn(a2, ra, -(float)s_s2[CT_BM + mm]), 0.f);
-                  const float b2 = __fmaf_rn(u, u, (float)(eps * eps));
-                  const float rb = rsqrtf(b2);
-                  const float val = b2 * rb;  // sqrt(u^2 + eps^2)
-                  obj += w * (val - eps);
-                  zc[j] += w * (val - eps);
-                  dd = w * (u * rb) * ra;  // w sigma'(s - s_ctg) / s
-                }
+                // mixed path: s = sqrt(F^2 + qmax2) and the soft-ReLU through reciprocal square
+                // roots (a few units in the last place, below the FP32 error of F itself)
+                float l0, l1;
+                unpack2(Lp[i >> 1][j], l0, l1);
+                Lx = (i & 1) ? l1 : l0;
+                Fx = F[i][j];
+                const float a2 = __fmaf_rn(F[i][j], F[i][j], (float)q2);
+                const float ra = rsqrtf(a2);
+                const float u = fmaxf(__fmaf_rn(a2, ra, -(float)s_s2[CT_BM + mm]), 0.f);
+                const float b2 = __fmaf_rn(u, u, (float)(eps * eps));
+                const float rb = rsqrtf(b2);
+                const float val = b2 * rb;  // sqrt(u^2 + eps^2)
+                obj += w * (val - eps);
+                zc[j] += w * (val - eps);
+                dd = w * (u * rb) * ra;  // w sigma'(s - s_ctg) / s
                 gm[i] += dd * Fx;
                 gk[j] += dd * Fx * Lx;
                 gq[i] += Real(0.5) * dd;     // dz/dqmax2 = w sigma' / (2 s)
