@@ -2578,18 +2578,17 @@ __device__ void s4_sdca(const Dev<Real, Dc> &d, const Inst &I, int tc, int sub) 
   if (lane == 0 && t < I.T) d.sp_part[(long long)sub * I.T + t] = s;
 }
 
-// Adjoint DC products and device updates of the dense DC mode (the last stage).  Warp w of the
-// block takes column c = sub * 8 + w of period t:
+// Adjoint DC products of the dense DC mode.  Column c of period t:
 //   eta'[t, c] = sum_m dz/df[t,m] A[c, m],   A[gb, m] = PTDF[m, gb] - (PTDF 1)[m] / n  (c = gb < Gb:
 //   the injection adjoint at generator bus gb minus its mean over all buses, Eqs. 2nd_lin_sys and
 //   correction, the mean folded into the column at set-up) | A[Gb + x, m] = PSDF[m, x] (transformer x,
-//   Eq. 2nd_lin_sys_phase),
-// lanes striding over the branches, a fixed-order shuffle reduction, and the sum broadcast to the
-// warp; then (mixed path) its lanes update the devices at the bus, one per lane, or lane 0 the
-// transformer (plans whose tab.fuse is set: small ones on the mixed path).  Otherwise the products are
-// stored for stage 5, which updates 32 (FP64 path) or 256 devices per block: the FP64 pipe takes
-// about as long for a warp with one active lane as for a full one, and large plans would get one
-// objective slot per stage-4 block.
+//   Eq. 2nd_lin_sys_phase).
+// s4_gbus (small plans on the mixed path, where stage 4 is the last): warp w of the block takes column
+// c = sub * 8 + w of period t, the sum is broadcast to the warp, and its lanes update the devices at the bus,
+// one per lane, or lane 0 the transformer.  gbus_column stores the products for stage 5, which updates 8 or 64
+// (FP64 path) or 256 devices per block: the FP64 pipe takes about as long for a warp with one active lane as
+// for a full one, and large plans would get one objective slot per stage-4 block.
+
 // Products of a column A (of I.M branches) with nt <= NT periods of dz/df, one warp: lanes stride over the
 // branches, four accumulators per period, a fixed-order shuffle reduction (each period's sum has the same order
 // whatever NT is); the sums are valid in lane 0.

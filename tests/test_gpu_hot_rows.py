@@ -54,3 +54,23 @@ def test_hot_rows_match_the_oracle(qg, precision, n, M, K, T, scale):
     assert abs(s.breakdown()[0, 7] - ref.terms["zctg"]) <= tol * abs(ref.terms["zctg"])
     check_prec(g.cpu().numpy(), ref.grad, c, precision, "hot rows")
     s.close()
+
+
+def test_hot_rows_screening_scores(qg):
+    """A screening handle: the scores of the selected outages hold the hot rows' share."""
+    c = grid(700, 1100, 998, 64)
+    c = dataclasses.replace(c, s_max_ctg=0.5 * c.s_max_ctg)
+    x = np.clip(synth.random_point(c, 3, 0.2), *oracle.box(c))
+    s = qg.Solver(c, precision=0, ctg_frac=0.5)
+    Ks = int(np.ceil(0.5 * c.K))
+    sel = np.sort(np.random.default_rng(1).choice(c.K, Ks, replace=False)).astype(np.int32)
+    qg.qg_ctg_select(s.h, 0, sel)
+    obj, g = s.eval_grad(torch.tensor(x, dtype=s.dtype, device="cuda"))
+    z = qg.qg_ctg_scores(s.h, c.T * Ks).reshape(c.T, Ks)
+    sub = dataclasses.replace(c, ctg=c.ctg[sel])
+    ref = oracle.evaluate(sub, x)
+    floor = c.dt[:, None] * c.c_s * c.beta * c.eps * (c.n_branch - 1)
+    assert abs(obj.item() - ref.obj) <= 1e-10 * abs(ref.obj)
+    assert np.max(np.abs(z - (ref.z_ctg - floor))) <= 1e-10 * np.abs(ref.z_ctg).max()
+    check_prec(g.cpu().numpy(), ref.grad, c, 0, "hot rows, screening")
+    s.close()
