@@ -1960,7 +1960,7 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
   gF += gk;
   if (lead) {
     // adjoints of the four end flows
-    const Real sf2 = sq_sum(pf, qf), st2 = sq_sum(pt, qt);
+    const Real sf2 = SPLIT > 1 ? sq_sum(qf, pf) : sq_sum(pf, qf), st2 = sq_sum(pt, qt);  // (each form's bits are kept)
     if (fmax(sf2, st2) > smax * smax) {  // thermal (Example 1)
       const Real sf = dsqrt(sf2), st = dsqrt(st2);
       const bool fr = sf >= st;
