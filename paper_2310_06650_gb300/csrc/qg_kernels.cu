@@ -1213,9 +1213,9 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
             const long long idx = I.tm0 + (long long)(t0 + tt) * I.M + m;
             f = d.f32[idx];
             qs = ctg_qs<Real>(d.qm2[idx], d.br_s2ctg[I.br0 + m]);
-            if (I.hot && row_hot(f, qs)) {  // s2_hot's row: F^2 - inf is never a candidate
+            if (I.hot && row_hot(f, qs)) {  // s2_hot's row, marked by a NaN: never a candidate
               f = 0.f;
-              qs = -INFINITY;
+              qs = f_nan();
             }
             if (F64) f64 = d.fre[idx];
           }
@@ -1247,7 +1247,7 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
             if (F64) f64 = d.fre[idx];
             if (I.hot && row_hot(f, qs)) {
               f = 0.f;
-              qs = -INFINITY;
+              qs = f_nan();
             } else {
               rmin = fminf(rmin, clear_margin(f, qs));
             }
@@ -1433,7 +1433,9 @@ __device__ void s2_ctg(const Dev<Real, Dc> &d, const Inst &I, int sub, Obj3<Dc> 
         for (int e = threadIdx.x; e < tn * CT_BM; e += NTHR) {
           const int tt = e / CT_BM, c = e % CT_BM, m = m0 + c;
           if (!s_hit[tt]) continue;
-          if (m < I.M && s_qs[(tc0 + tt) * CT_BM + c] != -INFINITY) {  // hot rows' partials are s2_hot's
+          // hot rows' partials are s2_hot's; their NaN q-terms mark them (no other row of a plan with hot rows has
+          // one: row_hot takes NaN for hot), every other row of the tile is written, unlimited ones (-inf) too
+          if (m < I.M && !(I.hot && isnan(s_qs[(tc0 + tt) * CT_BM + c]))) {
             const long long q = I.pm0 + ((long long)kt * T + t0 + tc0 + tt) * I.M + m;
             d.pm[q] = s_gm[e];
             d.pq[q] = s_gq[e];
