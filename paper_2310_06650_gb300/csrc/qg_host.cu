@@ -80,6 +80,7 @@ struct HostInst {
 
 struct qg_ctx {
   int n_inst = 0;
+  int device = -1;  // the GPU it was created on, which holds its arrays and runs its kernels
   qg_options opt{};
   std::vector<HostInst> hi;
   Plan plan{};
@@ -1273,6 +1274,7 @@ int check_device(qg_ctx *h) {
   if (cudaGetDeviceProperties(&p, dev) != cudaSuccess) return fail(h, QG_ERR_NO_DEVICE, "cudaGetDeviceProperties failed");
   if (p.major != 10 || p.minor != 3)
     return fail(h, QG_ERR_NO_DEVICE, std::string("libqg is built for sm_103a; device is ") + p.name);
+  h->device = dev;
   return QG_OK;
 }
 
@@ -1427,15 +1429,16 @@ bool overlap(const void *a, size_t na, const void *b, size_t nb) {
 }
 
 // Whether the stage kernels may write the caller's array p (n bytes of elements of size el) while an evaluation
-// reads x (nx bytes): aligned device memory apart from x.
-bool writable(const void *p, size_t n, size_t el, const void *x, size_t nx) {
+// reads x (nx bytes): aligned memory of the handle's own GPU, apart from x.  (Memory of another GPU needs peer
+// access in a kernel and none in a copy.)
+bool writable(const qg_ctx *h, const void *p, size_t n, size_t el, const void *x, size_t nx) {
   if ((uintptr_t)p % el || overlap(p, n, x, nx)) return false;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice;
+  return a.type == cudaMemoryTypeDevice && a.device == h->device;
 }
 
 // Closing kernel of n deferred iterations: the objective of the last one (read at its schedule
@@ -1777,8 +1780,8 @@ int qg_eval_grad(qg_ctx *h, const void *x, double *obj, void *g) {
   const size_t ng = rs * h->n_x, no = sizeof(double) * h->n_inst;
   // the last stages write the caller's arrays along with the handle's (rt617: two copies, 4 us of the 50);
   // arrays that a kernel must not write that early or cannot take a copy afterwards
-  const bool dg = g && writable(g, ng, rs, x, ng) && !overlap(g, ng, obj, no);
-  const bool dobj = obj && writable(obj, no, sizeof(double), x, ng) && !overlap(g, ng, obj, no);
+  const bool dg = g && writable(h, g, ng, rs, x, ng) && !overlap(g, ng, obj, no);
+  const bool dobj = obj && writable(h, obj, no, sizeof(double), x, ng) && !overlap(g, ng, obj, no);
   if (dg) bounds_register(g, ng);  // index-checked builds: the caller's arrays
   if (dobj) bounds_register(obj, no);
   int rc = run_eval(h, x, false, 0, 0, 0, nullptr, 0, nullptr, 0, 0, false, dobj ? obj : nullptr, dg ? g : nullptr);
