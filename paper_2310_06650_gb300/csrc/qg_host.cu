@@ -126,6 +126,16 @@ struct qg_ctx {
   std::string err;
 };
 
+bool qg::device_memory(const void *p, size_t el, int device) {
+  if ((uintptr_t)p % el) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 namespace {
 
 int fail(qg_ctx *h, int code, const std::string &msg) {
@@ -1429,16 +1439,9 @@ bool overlap(const void *a, size_t na, const void *b, size_t nb) {
 }
 
 // Whether the stage kernels may write the caller's array p (n bytes of elements of size el) while an evaluation
-// reads x (nx bytes): aligned memory of the handle's own GPU, apart from x.  (Memory of another GPU needs peer
-// access in a kernel and none in a copy.)
+// reads x (nx bytes): aligned memory of the handle's own GPU, apart from x.
 bool writable(const qg_ctx *h, const void *p, size_t n, size_t el, const void *x, size_t nx) {
-  if ((uintptr_t)p % el || overlap(p, n, x, nx)) return false;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return a.type == cudaMemoryTypeDevice && a.device == h->device;
+  return !overlap(p, n, x, nx) && device_memory(p, el, h->device);
 }
 
 // Closing kernel of n deferred iterations: the objective of the last one (read at its schedule

@@ -284,6 +284,10 @@ void bounds_unregister(const void *p);
 // 1: a checked access missed (line, address of the first); 0: none; -1: not an index-checked build.
 int bounds_report(long long *line, unsigned long long *addr);
 
+// Whether a kernel on `device` may write the caller's array p of elements of size el: aligned device memory of
+// that GPU.  (Memory of another GPU needs peer access in a kernel and none in a copy.)
+bool device_memory(const void *p, size_t el, int device);
+
 // One evaluation (with adam, the fused projected Adam update); with close, ended by the closing
 // kernel (the objective sum; step += 1 with adam), else the objective is left in the slots for a
 // later launch_finish.

@@ -30,7 +30,7 @@
 #include <string>
 #include <vector>
 
-#include "../../include/qg.h"
+#include "qg_internal.h"
 
 namespace {
 
@@ -618,6 +618,7 @@ long long pad8(long long n) { return (n + 7) / 8 * 8; }  // BF16 row strides: mu
 
 struct qg_mlp {
   int n_in, n_h, n_out, max_b;
+  int device = -1;  // the GPU it was created on
   long long ld_i, ld_h, ld_o, ld_b;  // padded BF16 row strides for rows of I, H, O and batch elements
   long long n_par;
   long long o_w1, o_b1, o_w2, o_b2, o_w3, o_b3;
@@ -793,6 +794,10 @@ int qg_mlp_create(qg_mlp **out, int32_t n_in, int32_t n_hidden, int32_t n_out, i
   if (cudaGetDeviceCount(&count) != cudaSuccess || count < 1) return mfail(nullptr, QG_ERR_NO_DEVICE, "no CUDA device");
   if (!tensor_map_encoder()) return mfail(nullptr, QG_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled is not available");
   qg_mlp *m = new qg_mlp();
+  if (cudaGetDevice(&m->device) != cudaSuccess) {
+    delete m;
+    return mfail(nullptr, QG_ERR_NO_DEVICE, "cudaGetDevice failed");
+  }
   m->n_in = n_in; m->n_h = n_hidden; m->n_out = n_out; m->max_b = max_batch;
   m->ld_i = pad8(n_in); m->ld_h = pad8(n_hidden); m->ld_o = pad8(n_out); m->ld_b = pad8(max_batch);
   m->o_w1 = 0; m->o_b1 = m->o_w1 + (long long)n_hidden * n_in;
@@ -801,7 +806,7 @@ int qg_mlp_create(qg_mlp **out, int32_t n_in, int32_t n_hidden, int32_t n_out, i
   m->n_par = m->o_b3 + n_out;
   const long long B = max_batch, H = n_hidden, I = n_in, O = n_out;
   const long long li = m->ld_i, lh = m->ld_h, lo = m->ld_o, lb = m->ld_b;
-  m->part_elems = std::max({64 * B * H, 64 * B * O, H * I, O * H, H * H});
+  m->part_elems = std::max({64 * B * H, 65 * B * O, H * I, O * H, H * H});  // 64 splits, and an output (qg_mlp_forward)
   int rc = 0;
   if ((rc = mal(m, &m->w, m->n_par)) || (rc = mal(m, &m->gw, m->n_par)) || (rc = mal(m, &m->am, m->n_par)) ||
       (rc = mal(m, &m->av, m->n_par)) || (rc = mal(m, &m->w1b, H * li)) || (rc = mal(m, &m->w2b, H * lh)) ||
@@ -854,10 +859,16 @@ int qg_mlp_forward(qg_mlp *m, const float *x, int32_t batch, float *y) {
   load_x(m, x, batch, false);
   const int sp = forward(m, batch);
   if (!sp) return QG_ERR_CUDA;
+  // y is written in place where a kernel may write it, else past the partial sums and copied
+  const long long ny = (long long)batch * m->n_out;
+  const bool direct = qg::device_memory(y, sizeof(float), m->device);
   EpiArgs a{};
-  a.P = m->part; a.B = batch; a.N = m->n_out; a.splits = sp; a.bias = m->w + m->o_b3; a.Z = y;
+  a.P = m->part; a.B = batch; a.N = m->n_out; a.splits = sp; a.bias = m->w + m->o_b3;
+  a.Z = direct ? y : m->part + sp * ny;
   epi<EPI_OUT, EPI_TC_O>(m, a);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess && !direct)
+    e = cudaMemcpyAsync(y, a.Z, sizeof(float) * ny, cudaMemcpyDeviceToDevice, m->stream);
   return e == cudaSuccess ? QG_OK : mfail(m, QG_ERR_CUDA, cudaGetErrorString(e));
 }
 

@@ -114,3 +114,16 @@ for prec, w in ((qg.QG_FP64, 8), (qg.QG_MIXED, 4)):
     for name, (hits, copies) in r.items():
         kernel = name.split(" ")[0] in ("own", "no")
         assert (hits > 0, copies) == ((True, 0) if kernel else (False, 1)), (name, hits, copies)
+
+
+def test_mlp_forward_writes_only_arrays_of_its_own_gpu(child):
+    r = child(r"""
+m = qg.qg_mlp_create(65, 33, 127, 7)
+for B in (7, 1):
+    x, y, far, man = Buf(4 * 65 * 7), Buf(4 * 127 * 7 + 64), Buf(4 * 127 * 7, 1), Buf(4 * 127 * 7, 0, MANAGED)
+    for name, out in (("own", y), ("other gpu", far), ("managed", man), ("misaligned", y.at(2))):
+        res[f"{name} {B}"] = routed(out, lambda: qg.qg_mlp_forward(m, x, B, out))
+qg.qg_mlp_destroy(m)
+""")
+    for name, (hits, copies) in r.items():
+        assert (hits, copies) == ((1, 0) if name.startswith("own") else (0, 1)), (name, hits, copies)
