@@ -922,6 +922,10 @@ int build_tail(qg_ctx *h, Dev<Real, Dc> &d, const HostInst &H) {
     return rc;
   m.part = part;
   d.tail = &m;
+  if (split_prepare(S) != cudaSuccess) {
+    cudaGetLastError();  // a refused attribute is not a sticky error
+    return fail(h, QG_ERR_UNSUPPORTED, "the tail product's shared memory is not available on this device");
+  }
   if (!split_maps(m, S)) return fail(h, QG_ERR_UNSUPPORTED, "the driver's TMA descriptor encoder is not available");
   double *src;
   if ((rc = upload(h, &src, H.sinv))) return rc;

@@ -463,16 +463,6 @@ cudaError_t launch(void (*kern)(KArgs...), dim3 grid, int block, size_t smem, cu
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-template <int S>
-cudaError_t prepare() {
-  static std::once_flag once;
-  static cudaError_t e = cudaSuccess;
-  std::call_once(once, [] {
-    e = cudaFuncSetAttribute(k_split_gemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_smem_bytes<S>());
-  });
-  return e;
-}
-
 PFN_cuTensorMapEncodeTiled_v12000 encoder() {
   static std::once_flag once;
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -510,6 +500,12 @@ bool split_maps(SplitMat &m, int digits) {
   return encode(&m.ta, m.a, 2, da, sa, ba) && encode(&m.tb, m.b, 3, db, sb, bb);
 }
 
+cudaError_t split_prepare(int digits) {
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  return digits == 8 ? cudaFuncSetAttribute(k_split_gemm<8>, attr, (int)split_smem_bytes<8>())
+                     : cudaFuncSetAttribute(k_split_gemm<7>, attr, (int)split_smem_bytes<7>());
+}
+
 cudaError_t split_matrix(const SplitMat &m, const double *src, int digits, cudaStream_t s) {
   if (digits == 8) k_split_rows<8><<<m.rows, 256, 0, s>>>(src, m.K, m.a, m.ascale);
   else k_split_rows<7><<<m.rows, 256, 0, s>>>(src, m.K, m.a, m.ascale);
@@ -525,11 +521,9 @@ cudaError_t split_rhs(const SplitMat &m, const Dc *z, cudaStream_t s, bool pdl) 
 template <typename Dc>
 cudaError_t split_product(const SplitMat &m, const SplitOut<Dc> &out, cudaStream_t s, bool pdl) {
   constexpr int S = split_digits<Dc>();
-  cudaError_t e = prepare<S>();
   const int n_rt = (m.rows + SPLIT_ROWS - 1) / SPLIT_ROWS;
-  if (e == cudaSuccess)
-    e = launch(k_split_gemm<S>, dim3(n_rt * m.ks), SPLIT_THREADS, split_smem_bytes<S>(), s, pdl, m.ta, m.tb, (longlong2 *)m.part,
-               n_rt, m.K, m.T, m.nt, m.ks, m.kbps);
+  cudaError_t e = launch(k_split_gemm<S>, dim3(n_rt * m.ks), SPLIT_THREADS, split_smem_bytes<S>(), s, pdl, m.ta, m.tb,
+                         (longlong2 *)m.part, n_rt, m.K, m.T, m.nt, m.ks, m.kbps);
   if (e == cudaSuccess)
     e = launch(k_split_sum<Dc, S>, dim3((m.rows + 31) / 32, (m.T + SUM_T - 1) / SUM_T), 32 * SUM_T, 0, s, pdl,
                (const longlong2 *)m.part, (const float *)m.ascale, (const float *)m.bscale, m.rows, m.T, m.ks, n_rt, out);

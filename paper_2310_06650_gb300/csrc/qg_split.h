@@ -47,6 +47,10 @@ long long split_elems(const SplitMat &m, int digits);
 // Tensor maps of m (whose sizes and buffers are set); false when the driver's encoder is missing or refuses.
 bool split_maps(SplitMat &m, int digits);
 
+// Raises the product kernel's shared-memory limit on the current GPU (the limit belongs to a function on one
+// device): once for each matrix, before its first product.
+cudaError_t split_prepare(int digits);
+
 // Digits of A from its FP64 rows (device array, row stride K); digits = 7 or 8.
 cudaError_t split_matrix(const SplitMat &m, const double *src, int digits, cudaStream_t s);
 

@@ -2,7 +2,7 @@
 with a fake CUDA runtime (fake_cudart.cpp, where "device" memory is host memory with a device ordinal and
 kernels do not run) in a child process.
 
-Outputs: a kernel may write the caller's array only if it is aligned memory of the handle's own GPU apart
+Limits: shared memory above 48 KB has to be granted on each GPU.  Outputs: a kernel may write the caller's array only if it is aligned memory of the handle's own GPU apart
 from the inputs; every other array takes a copy after the kernels, as it did when all of them did."""
 import json
 import os
@@ -127,3 +127,20 @@ qg.qg_mlp_destroy(m)
 """)
     for name, (hits, copies) in r.items():
         assert (hits, copies) == ((1, 0) if name.startswith("own") else (0, 1)), (name, hits, copies)
+
+
+def test_sparse_handles_evaluate_on_every_gpu(child):
+    """The tail product's shared-memory limit is an attribute of its kernel on one GPU."""
+    r = child(r"""
+c = synth.make_case("tail", 617, 925, 88, T=3, K=20, seed=1)
+for dev in (0, 1):
+    fake.fake_set_device(dev)
+    for prec, w in ((qg.QG_FP64, 8), (qg.QG_MIXED, 4)):
+        h = handle(c, prec, dc_solver=qg.QG_DC_SPARSE)
+        x, obj, g = Buf(w * qg.qg_num_vars(h), dev), Buf(8, dev), Buf(w * qg.qg_num_vars(h), dev)
+        for _ in range(2):
+            qg.qg_eval_grad(h, x, obj, g)
+        qg.qg_destroy(h)
+        res[f"{dev} {prec}"] = True
+""")
+    assert len(r) == 4
