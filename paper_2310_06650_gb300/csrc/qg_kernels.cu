@@ -3110,17 +3110,22 @@ cudaError_t launch_eval(const Dev<Real, Dc> &d, const Plan &P, const void *x, bo
                            : launch_stages<Real, Dc, MAXB>(d, P, x, adam, close, s, ev);
 }
 
-// The contingency kernel's dynamic shared-memory limit is a process-wide function attribute: it is
-// only ever raised, so that creating a handle with smaller blocks never breaks an existing one.
+// The contingency kernel's dynamic shared-memory limit is an attribute of the function on one device, shared
+// by that device's handles: it is only ever raised, so that creating a handle with smaller blocks never
+// breaks an existing one.
 template <typename Real, typename Dc>
 cudaError_t prepare_eval(int maxTB, bool score, bool lazy, bool hot) {
+  constexpr int MAX_DEVICES = 64;
   static std::mutex mu;
-  static size_t cur = 0;  // the same limit for every instantiation
+  static size_t cur[MAX_DEVICES] = {};  // per device; the same limit for every instantiation
   const size_t sm = ctg_smem_bytes<Real>(maxTB, score, lazy, hot);
   if (sm > 227 * 1024) return cudaErrorInvalidValue;
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
-  if (sm <= cur) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
+  if (sm <= cur[dev]) return cudaSuccess;
   auto raise = [&](auto kern) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   };
@@ -3130,7 +3135,7 @@ cudaError_t prepare_eval(int maxTB, bool score, bool lazy, bool hot) {
   raise(k_s2<Real, Dc, 0, MAXB>);
   raise(k_s2<Real, Dc, 1, MAXB>);
   raise(k_s2<Real, Dc, 2, MAXB>);
-  if (e == cudaSuccess) cur = sm;
+  if (e == cudaSuccess) cur[dev] = sm;
   return e;
 }
 

@@ -144,3 +144,22 @@ for dev in (0, 1):
         res[f"{dev} {prec}"] = True
 """)
     assert len(r) == 4
+
+
+def test_contingency_blocks_evaluate_on_every_gpu(child):
+    """A contingency block of many periods (above 48 KB on both paths), then a smaller one, on the first GPU
+    and then on the second."""
+    r = child(r"""
+big, small = synth.make_case("big", 90, 140, 9, T=48, K=20, seed=1), synth.mid()
+for dev in (0, 1):
+    fake.fake_set_device(dev)
+    for prec, w in ((qg.QG_FP64, 8), (qg.QG_MIXED, 4)):
+        hs = [handle(c, prec, ctg_bound=qg.QG_CTG_BOUND_LAZY) for c in (big, small)]
+        for h in hs:
+            n = qg.qg_num_vars(h)
+            qg.qg_eval_grad(h, Buf(w * n, dev), Buf(8, dev), Buf(w * n, dev))
+        for h in hs:
+            qg.qg_destroy(h)
+        res[f"{dev} {prec}"] = True
+""")
+    assert len(r) == 4
