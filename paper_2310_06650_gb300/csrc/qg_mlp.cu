@@ -686,15 +686,11 @@ int make_map(qg_mlp *m, CUtensorMap *map, const __nv_bfloat16 *ptr, long long ro
   return QG_OK;
 }
 
+// Raises the kernel's shared-memory limit on the current GPU (the limit belongs to a function on one device).
 template <int BN, int STAGES>
 cudaError_t umma_prepare() {
-  static std::once_flag once;
-  static cudaError_t e = cudaSuccess;
-  std::call_once(once, [] {
-    e = cudaFuncSetAttribute(k_umma_gemm<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)umma_smem_bytes<BN, STAGES>());
-  });
-  return e;
+  return cudaFuncSetAttribute(k_umma_gemm<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)umma_smem_bytes<BN, STAGES>());
 }
 
 // Split-K partials of C = A B^T (A: M x K with row stride lda, B: N x K with row stride ldb, both BF16)
@@ -720,15 +716,11 @@ int gemm(qg_mlp *mm, const __nv_bfloat16 *A, long long lda, int M, const __nv_bf
   float *out = dst ? dst : mm->part;
   cudaError_t e;
   if (narrow) {
-    e = umma_prepare<64, 4>();
-    if (e == cudaSuccess)
-      e = pdl_launch(k_umma_gemm<64, 4>, grid, dim3(UTHREADS), umma_smem_bytes<64, 4>(), mm->stream, ta, tb, out, M,
-                     N, nkb, kbps, trans ? 1 : 0, a_static ? 1 : 0, mm->d_err);
+    e = pdl_launch(k_umma_gemm<64, 4>, grid, dim3(UTHREADS), umma_smem_bytes<64, 4>(), mm->stream, ta, tb, out, M,
+                   N, nkb, kbps, trans ? 1 : 0, a_static ? 1 : 0, mm->d_err);
   } else {
-    e = umma_prepare<256, 2>();
-    if (e == cudaSuccess)
-      e = pdl_launch(k_umma_gemm<256, 2>, grid, dim3(UTHREADS), umma_smem_bytes<256, 2>(), mm->stream, ta, tb, out,
-                     M, N, nkb, kbps, trans ? 1 : 0, a_static ? 1 : 0, mm->d_err);
+    e = pdl_launch(k_umma_gemm<256, 2>, grid, dim3(UTHREADS), umma_smem_bytes<256, 2>(), mm->stream, ta, tb, out,
+                   M, N, nkb, kbps, trans ? 1 : 0, a_static ? 1 : 0, mm->d_err);
   }
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -820,6 +812,14 @@ int qg_mlp_create(qg_mlp **out, int32_t n_in, int32_t n_hidden, int32_t n_out, i
     qg_mlp_destroy(m);
     return rc;
   }
+  cudaError_t e = umma_prepare<64, 4>();
+  if (e == cudaSuccess) e = umma_prepare<256, 2>();
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // a refused attribute is not a sticky error
+    mfail(m, QG_ERR_CUDA, std::string("tensor-core GEMM launch: ") + cudaGetErrorString(e));
+    qg_mlp_destroy(m);
+    return QG_ERR_CUDA;
+  }
   cudaMemset(m->gw, 0, m->n_par * sizeof(float));
   cudaMemset(m->am, 0, m->n_par * sizeof(float));
   cudaMemset(m->av, 0, m->n_par * sizeof(float));
@@ -830,7 +830,7 @@ int qg_mlp_create(qg_mlp **out, int32_t n_in, int32_t n_hidden, int32_t n_out, i
   k_init<<<grid_for(H * H), 256>>>(m->w + m->o_w2, H * H, sqrtf(2.f / (float)H), seed, H * I);
   k_init<<<grid_for(O * H), 256>>>(m->w + m->o_w3, O * H, sqrtf(1.f / (float)H), seed, H * I + H * H);
   refresh_bf16(m);
-  cudaError_t e = cudaDeviceSynchronize();
+  e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     mfail(m, QG_ERR_CUDA, std::string("init: ") + cudaGetErrorString(e));
     qg_mlp_destroy(m);

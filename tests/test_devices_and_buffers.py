@@ -163,3 +163,17 @@ for dev in (0, 1):
         res[f"{dev} {prec}"] = True
 """)
     assert len(r) == 4
+
+
+def test_networks_run_on_every_gpu(child):
+    r = child(r"""
+for dev in (0, 1):
+    fake.fake_set_device(dev)
+    m = qg.qg_mlp_create(65, 33, 127, 7)
+    x, t, y = Buf(4 * 65 * 7, dev), Buf(4 * 127 * 7, dev), Buf(4 * 127 * 7, dev)
+    qg.qg_mlp_forward(m, x, 7, y)
+    qg.qg_mlp_train_step(m, x, t, 7, 1e-3)
+    qg.qg_mlp_destroy(m)
+    res[str(dev)] = True
+""")
+    assert len(r) == 2
