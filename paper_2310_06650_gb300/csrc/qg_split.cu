@@ -18,6 +18,7 @@
 
 #include "qg_internal.h"
 #include "qg_split.h"
+#include "qg_split_feed.h"
 
 namespace qg {
 namespace {
@@ -152,7 +153,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   unsigned char *sA = base, *sB = base + SPLIT_STAGES * A_BYTES;
   __shared__ __align__(8) uint64_t fullA[SPLIT_STAGES], emptyA[SPLIT_STAGES], fullB[2], emptyB[2], accf, acce, drain;
   __shared__ uint32_t s_tmem;
-  __shared__ int s_abort, s_issued;
+  __shared__ int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rt = blockIdx.x / ks, kp = blockIdx.x % ks;
   const int nkb_all = (K + SPLIT_KB - 1) / SPLIT_KB;
@@ -172,7 +173,6 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
     mbar_init(&drain, 1);
     mbar_init(&acce, SPLIT_EPI / 32);
     s_abort = 0;
-    s_issued = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -189,35 +189,36 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   const int nch = (nkb + KB_PER_CHUNK - 1) / KB_PER_CHUNK;
   if (warp == 8) {
     if (lane == 0) {  // producer: A's digits are static, B's wait for the kernel before
-      int n = 0;      // A tiles requested so far
-      bool ok = true;
-      for (int p = 0; p < passes && ok; ++p)
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-          const int u = p * nkb + kb, kx = (kb0 + kb) * SPLIT_KB;  // a multiple of 64 elements: 128-byte aligned
-          for (int i = 0; i < S && ok; ++i, ++n) {
-            const int st = n % SPLIT_STAGES;
-            if (n >= SPLIT_STAGES && !mbar_wait(&emptyA[st], (uint32_t)(n / SPLIT_STAGES - 1) & 1, abort, true)) {
-              ok = false;
-              break;
-            }
-            mbar_expect_tx(&fullA[st], A_BYTES);
-            tma_load_2d(sA + st * A_BYTES, &tA, &fullA[st], 0, ((rt * nkb_all + kb0 + kb) * S + i) * SPLIT_ROWS);
-            if (i == 0) {  // after the first A tile, so that this one is in flight during the wait
-              if (u == 0) wait_grid();
-              if (u >= 2 && !mbar_wait(&emptyB[u & 1], (uint32_t)(u / 2 - 1) & 1, abort, true)) {
-                ok = false;
-                ++n;
-                break;
-              }
-              mbar_expect_tx(&fullB[u & 1], b_bytes);
-              tma_load_3d(sB + (u & 1) * (size_t)b_bytes, &tB, &fullB[u & 1], kx, p * nt, 0);
-            }
-          }
-          if (ok) s_issued = u + 1;
+      struct {
+        const CUtensorMap &tA, &tB;
+        unsigned char *sA, *sB;
+        uint64_t *fullA, *emptyA, *fullB, *emptyB;
+        volatile int *abort;
+        uint32_t b_bytes;
+        int nt, nkb, kb0, tile0;  // K blocks of the block, the first, and its tile of digit 0
+        int p, kb;                // pass and K block of the unit
+        __device__ bool wait_a_free(int n) const {
+          return mbar_wait(&emptyA[n % SPLIT_STAGES], (uint32_t)(n / SPLIT_STAGES - 1) & 1, abort, true);
         }
-      // drain: every copy requested has landed before the block may exit (bounded waits)
-      for (int q = max(0, n - SPLIT_STAGES); q < n; ++q)
-        mbar_wait(&fullA[q % SPLIT_STAGES], (uint32_t)(q / SPLIT_STAGES) & 1, abort, false);
+        __device__ bool wait_b_free(int u) const { return mbar_wait(&emptyB[u & 1], (uint32_t)(u / 2 - 1) & 1, abort, true); }
+        __device__ void wait_inputs() const { wait_grid(); }
+        __device__ void load_a(int n, int u, int i) {
+          if (i == 0 && u > 0 && ++kb == nkb) {
+            kb = 0;
+            ++p;
+          }
+          const int st = n % SPLIT_STAGES;
+          mbar_expect_tx(&fullA[st], A_BYTES);
+          tma_load_2d(sA + st * A_BYTES, &tA, &fullA[st], 0, ((tile0 + kb) * S + i) * SPLIT_ROWS);
+        }
+        __device__ void load_b(int u) const {  // from a multiple of 64 elements: 128-byte aligned
+          mbar_expect_tx(&fullB[u & 1], b_bytes);
+          tma_load_3d(sB + (u & 1) * (size_t)b_bytes, &tB, &fullB[u & 1], (kb0 + kb) * SPLIT_KB, p * nt, 0);
+        }
+        __device__ void drain_a(int q) const { mbar_wait(&fullA[q % SPLIT_STAGES], (uint32_t)(q / SPLIT_STAGES) & 1, abort, false); }
+        __device__ void drain_b(int u) const { mbar_wait(&fullB[u & 1], (uint32_t)(u / 2) & 1, abort, false); }
+      } ops{tA, tB, sA, sB, fullA, emptyA, fullB, emptyB, abort, b_bytes, nt, nkb, kb0, rt * nkb_all + kb0, 0, 0};
+      split_feed<SPLIT_STAGES>(ops, passes * nkb, S);
     }
   } else if (warp == 9) {
     if (lane == 0) {  // MMA issuer
@@ -311,8 +312,6 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (warp == 8 && lane == 0)  // after an abort: the B copies requested and not consumed
-    for (int u = max(0, s_issued - 2); u < s_issued; ++u) mbar_wait(&fullB[u & 1], (uint32_t)(u / 2) & 1, abort, false);
   if (warp == 9) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
