@@ -917,7 +917,7 @@ int build_tail(qg_ctx *h, Dev<Real, Dc> &d, const HostInst &H) {
   int rc;
   longlong2 *part;
   if ((rc = dalloc(h, &m.a, (size_t)split_elems(m, S))) || (rc = dalloc(h, &m.b, (size_t)S * m.T * m.ld)) ||
-      (rc = dalloc(h, &m.ascale, (size_t)m.rows)) || (rc = dalloc(h, &m.bscale, (size_t)m.T)) ||
+      (rc = dalloc(h, &m.aexp, (size_t)m.rows)) || (rc = dalloc(h, &m.bexp, (size_t)m.T)) ||
       (rc = dalloc(h, &part, (size_t)m.ks * n_rt * SPLIT_ROWS * m.T)))
     return rc;
   m.part = part;

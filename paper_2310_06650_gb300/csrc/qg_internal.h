@@ -201,7 +201,7 @@ struct Dev {
   Dc *sp_rhs, *sp_u, *sp_th, *sp_zt;  // [nr T], [nr T], [nr T], [nT T]
   Dc *sp_mu;                          // [T] mean injection (uniform slack)
   Dc *sp_part;                        // [n_pchunk][T] partial sums of z1 . w
-  unsigned int *sp_bmax;              // [2][SPLIT_SPREAD][T] largest |z_T| per period, forward and adjoint solve (bits)
+  unsigned int *sp_bmax;              // [2][SPLIT_SPREAD][T] largest split_key of z_T per period, forward and adjoint solve
   // penalty parameters
   Real c_p, c_q, c_s, c_rz, rho, eps, beta;
   double c_s64, eps64, beta64;        // the same options in FP64 (closed-form objective floor)

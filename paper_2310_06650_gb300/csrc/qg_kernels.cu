@@ -197,9 +197,6 @@ struct DcOps<df32> {
   __device__ static df32 bcast(df32 a) { return {__shfl_sync(0xffffffffu, a.hi, 0), __shfl_sync(0xffffffffu, a.lo, 0)}; }
 };
 
-// |a| rounded up to FP32
-__device__ __forceinline__ float abs_up(double a) { return __double2float_ru(fabs(a)); }
-__device__ __forceinline__ float abs_up(df32 a) { return __fadd_ru(fabsf(a.hi), fabsf(a.lo)); }
 __device__ __forceinline__ double to_double(double a) { return a; }
 __device__ __forceinline__ double to_double(df32 a) { return (double)a.hi + (double)a.lo; }
 
@@ -2875,11 +2872,11 @@ __global__ void __launch_bounds__(NTHR) k_sp_fwd(const __grid_constant__ Dev<Rea
         unsigned *mx = d.sp_bmax + ((ADJ ? SPLIT_SPREAD : 0) + row % SPLIT_SPREAD) * T;
         if (ta < T) {
           z[ta] = z0 = DcOps<Dc>::add(b[ta], z0);
-          atomicMax(mx + ta, __float_as_uint(abs_up(z0)));
+          atomicMax(mx + ta, split_key(z0));
         }
         if (tb < T) {
           z[tb] = z1 = DcOps<Dc>::add(b[tb], z1);
-          atomicMax(mx + tb, __float_as_uint(abs_up(z1)));
+          atomicMax(mx + tb, split_key(z1));
         }
       }
       __syncthreads();

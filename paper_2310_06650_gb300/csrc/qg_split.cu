@@ -29,6 +29,7 @@ constexpr int SPLIT_EPI = 256;                  // epilogue threads (warps 0-7)
 constexpr int SPLIT_THREADS = SPLIT_EPI + 64;   // + TMA producer warp, MMA warp
 constexpr unsigned long long SPLIT_WAIT_NS = 1000000000ull;  // a wait gives up after 1 s (NaN results, clean exit)
 constexpr long long SPLIT_LOST = 1ll << 62;  // a block's partial sums after a wait ran out (real ones are below 2^61)
+constexpr int SPLIT_NONFINITE = 1 << 20;  // in place of an exponent: an operand is infinite or NaN
 constexpr uint32_t A_BYTES = SPLIT_ROWS * SPLIT_KB * 2;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -125,20 +126,20 @@ constexpr size_t split_smem_bytes() {
   return (size_t)SPLIT_STAGES * A_BYTES + 2 * (size_t)S * SPLIT_NT * SPLIT_KB * 2 + 1024;
 }
 
-// The finished value of two 64-bit sums: hi 2^-24 + lo 2^-(24 + 8 (S - 4)), times 2^(ea + eb - 12).
+// The finished value of two 64-bit sums: hi 2^-24 + lo 2^-(24 + 8 (S - 4)), times 2^(e - 12) with e the sum of the
+// two operands' exponents.
 template <int S>
-__device__ __forceinline__ double split_value(long long hi, long long lo, float sa, float sb, double) {
+__device__ __forceinline__ double split_value(long long hi, long long lo, int e, double) {
   constexpr double W = S == 8 ? 0x1p-32 : 0x1p-24;
-  return (((double)hi + (double)lo * W) * ((double)sa * 0x1p-36)) * (double)sb;
+  return scalbn((double)hi + (double)lo * W, e - 36);
 }
 template <int S>
-__device__ __forceinline__ df32 split_value(long long hi, long long lo, float sa, float sb, df32) {
+__device__ __forceinline__ df32 split_value(long long hi, long long lo, int e, df32) {
   constexpr float W = S == 8 ? 0x1p-32f : 0x1p-24f;
   const float h = (float)hi;
   const float l = (float)(hi - (long long)h) + (float)lo * W;
-  const float s = __fadd_rn(h, l), e = __fadd_rn(l, __fsub_rn(h, s));
-  const float k = sa * 0x1p-36f;
-  return {s * k * sb, e * k * sb};
+  const float s = __fadd_rn(h, l), r = __fadd_rn(l, __fsub_rn(h, s));
+  return {scalbnf(s, e - 36), scalbnf(r, e - 36)};
 }
 
 __device__ __forceinline__ double dc_nan(double) { return nan(""); }
@@ -323,19 +324,19 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
 constexpr int SUM_T = 8;
 
 template <typename Dc, int S>
-__global__ void __launch_bounds__(32 * SUM_T) k_split_sum(const longlong2 *__restrict__ part, const float *__restrict__ ascale,
-                                                         const float *__restrict__ bscale, int rows, int T, int ks,
+__global__ void __launch_bounds__(32 * SUM_T) k_split_sum(const longlong2 *__restrict__ part, const int *__restrict__ aexp,
+                                                         const int *__restrict__ bexp, int rows, int T, int ks,
                                                          int n_rt, const __grid_constant__ SplitOut<Dc> out) {
   __shared__ Dc s_v[32][SUM_T + 1];
   const int r0 = blockIdx.x * 32, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int t0 = blockIdx.y * SUM_T, tn = min(SUM_T, T - t0);
-  const float sa = ascale[min(r0 + lane, rows - 1)];
+  const int ea = aexp[min(r0 + lane, rows - 1)];
   wait_grid();
   const int t = min(t0 + wid, T - 1);
   const longlong2 *src = part + ((long long)(r0 / SPLIT_ROWS) * T + t) * SPLIT_ROWS + r0 % SPLIT_ROWS + lane;
-  const float sb = bscale[t];
+  const int eb = bexp[t];
   long long hi = 0, lo = 0;
-  bool lost = false;
+  bool lost = ea == SPLIT_NONFINITE || eb == SPLIT_NONFINITE;
 #pragma unroll 8
   for (int q = 0; q < ks; ++q) {
     const longlong2 v = src[(long long)q * n_rt * T * SPLIT_ROWS];
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(32 * SUM_T) k_split_sum(const longlong2 *__res
     hi += v.x;
     lo += v.y;
   }
-  s_v[lane][wid] = lost ? dc_nan(Dc{}) : split_value<S>(hi, lo, sa, sb, Dc{});
+  s_v[lane][wid] = lost ? dc_nan(Dc{}) : split_value<S>(hi, lo, ea + eb, Dc{});
   __syncthreads();
   const int r = threadIdx.x / SUM_T, tt = threadIdx.x % SUM_T, pos = out.pos0 + r0 + r;
   if (r0 + r >= rows || tt >= tn) return;
@@ -356,15 +357,16 @@ __global__ void __launch_bounds__(32 * SUM_T) k_split_sum(const longlong2 *__res
   }
 }
 
-// A power of two 2^e > m (its exponent field, one up), at least 2^-87 so that 2^54 / 2^e stays within FP32's
-// range (smaller operands lose bits below 2^-141); NaN for an infinity or NaN.
-__device__ __forceinline__ float pow2_above(float m) {
-  if (!(m < INFINITY)) return __int_as_float(0x7fc00000);
-  const unsigned f = __float_as_uint(m) >> 23;
-  return __uint_as_float(min(max(f + 1, 40u), 253u) << 23);
+// The exponent e with m < 2^e of the operands whose largest magnitude m has the key (split_key), over the whole
+// range of the type; SPLIT_NONFINITE where there is an infinity or NaN.
+__device__ __forceinline__ int split_exp(unsigned key, double) {
+  return key >= 0x7ff00000u ? SPLIT_NONFINITE : max((int)(key >> 20), 1) - 1022;
+}
+__device__ __forceinline__ int split_exp(unsigned key, df32) {
+  return key >= 0x7f800000u ? SPLIT_NONFINITE : max((int)(key >> 23), 1) - 126;
 }
 
-// Digit i of x (the value times 2^(8 S - 2) / 2^e, |x| < 2^(8 S - 2)), most significant first.
+// Digit i of x (the value times 2^(8 S - 2 - e), |x| <= 2^(8 S - 2)), most significant first.
 template <int S>
 __device__ __forceinline__ void digits(long long x, float (&q)[S]) {
 #pragma unroll
@@ -376,48 +378,52 @@ __device__ __forceinline__ void digits(long long x, float (&q)[S]) {
   q[0] = (float)(int)x;
 }
 
+// v 2^n as an integer, in two steps within the type's range (exact down to what rounds to zero).
+__device__ __forceinline__ long long fixed_point(double v, int n) {
+  const int h = n >> 1;
+  return __double2ll_rn(v * __hiloint2double((h + 1023) << 20, 0) * __hiloint2double((n - h + 1023) << 20, 0));
+}
+__device__ __forceinline__ long long fixed_point(df32 v, int n) {
+  const int h = n >> 1;
+  const float k1 = __int_as_float((h + 127) << 23), k2 = __int_as_float((n - h + 127) << 23);
+  return __float2ll_rn(v.hi * k1 * k2) + __float2ll_rn(v.lo * k1 * k2);
+}
+
 // Set-up: digits of one row of A per block, into the tiles [row tile][K block][digit][128][64] (whose pads stay 0).
 template <int S>
 __global__ void __launch_bounds__(256) k_split_rows(const double *__restrict__ src, int K, __nv_bfloat16 *__restrict__ a,
-                                                    float *__restrict__ scale) {
-  __shared__ float red[8];
-  __shared__ float s_sc;
+                                                    int *__restrict__ aexp) {
+  __shared__ unsigned red[8];
+  __shared__ int s_e;
   const double *row = src + (long long)blockIdx.x * K;
-  float mx = 0.f;
-  for (int k = threadIdx.x; k < K; k += 256) mx = fmaxf(mx, __double2float_ru(fabs(row[k])));
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  unsigned mx = 0;
+  for (int k = threadIdx.x; k < K; k += 256) mx = max(mx, split_key(row[k]));
+  mx = __reduce_max_sync(0xffffffffu, mx);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) mx = fmaxf(mx, red[w]);
-    s_sc = pow2_above(mx);
-    scale[blockIdx.x] = s_sc;
+    for (int w = 1; w < 8; ++w) mx = max(mx, red[w]);
+    s_e = split_exp(mx, 0.0);
+    aexp[blockIdx.x] = s_e;
   }
   __syncthreads();
-  const double k2 = ldexp(1.0, 8 * S - 2) / (double)s_sc;
   const int rt = blockIdx.x / SPLIT_ROWS, r = blockIdx.x % SPLIT_ROWS, nkb = (K + SPLIT_KB - 1) / SPLIT_KB;
   for (int k = threadIdx.x; k < K; k += 256) {
     float q[S];
-    digits<S>(__double2ll_rn(row[k] * k2), q);
+    digits<S>(s_e != SPLIT_NONFINITE ? fixed_point(row[k], 8 * S - 2 - s_e) : 0ll, q);
     __nv_bfloat16 *dst = a + (((long long)(rt * nkb + k / SPLIT_KB) * S) * SPLIT_ROWS + r) * SPLIT_KB + k % SPLIT_KB;
 #pragma unroll
     for (int i = 0; i < S; ++i) dst[(long long)i * SPLIT_ROWS * SPLIT_KB] = __float2bfloat16_rn(q[i]);
   }
 }
 
-__device__ __forceinline__ long long fixed_point(double v, float sc, double) { return __double2ll_rn(v * (0x1p62 / (double)sc)); }
-__device__ __forceinline__ long long fixed_point(df32 v, float sc, df32) {  // 2^54 / 2^e: within FP32's range in two steps
-  const float k = 0x1p27f / sc;
-  return __float2ll_rn(v.hi * k * 0x1p27f) + __float2ll_rn(v.lo * k * 0x1p27f);
-}
-
 // Digits of the right-hand sides: 64 rows x SPLIT_RT columns of z [K][T] per block, turned to [digit][t][k] through shared memory.
 template <typename Dc, int S>
 __global__ void __launch_bounds__(256) k_split_rhs(const Dc *__restrict__ z, int K, int T, __nv_bfloat16 *__restrict__ b, long long ld,
                                                    long long slice, const unsigned *__restrict__ bmax,
-                                                   float *__restrict__ scale) {
+                                                   int *__restrict__ bexp) {
   __shared__ Dc s_z[SPLIT_KB][SPLIT_RT + 1];
-  __shared__ float s_sc[SPLIT_RT];
+  __shared__ int s_e[SPLIT_RT];
   const int k0 = blockIdx.x * SPLIT_KB, kn = min(SPLIT_KB, K - k0), lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   wait_grid();
   const int t0 = blockIdx.y * SPLIT_RT, tn = min(SPLIT_RT, T - t0);
@@ -429,16 +435,17 @@ __global__ void __launch_bounds__(256) k_split_rhs(const Dc *__restrict__ z, int
     unsigned m = 0;
 #pragma unroll
     for (int q = 0; q < SPLIT_SPREAD; ++q) m = max(m, bmax[q * T + t0 + threadIdx.x]);
-    s_sc[threadIdx.x] = pow2_above(__uint_as_float(m));
-    if (blockIdx.x == 0) scale[t0 + threadIdx.x] = s_sc[threadIdx.x];
+    s_e[threadIdx.x] = split_exp(m, Dc{});
+    if (blockIdx.x == 0) bexp[t0 + threadIdx.x] = s_e[threadIdx.x];
   }
   __syncthreads();
   for (int t = wid; t < tn; t += 8) {  // lanes: pairs of consecutive k, one 128-byte line per (digit, t)
-    const float sc = s_sc[t];
+    const bool ok = s_e[t] != SPLIT_NONFINITE;
+    const int n = 8 * S - 2 - s_e[t];
     float q0[S], q1[S];
     const int k = 2 * lane;
-    digits<S>(k < kn && sc == sc ? fixed_point(s_z[k][t], sc, Dc{}) : 0ll, q0);
-    digits<S>(k + 1 < kn && sc == sc ? fixed_point(s_z[k + 1][t], sc, Dc{}) : 0ll, q1);
+    digits<S>(k < kn && ok ? fixed_point(s_z[k][t], n) : 0ll, q0);
+    digits<S>(k + 1 < kn && ok ? fixed_point(s_z[k + 1][t], n) : 0ll, q1);
     if (k0 + k < (int)ld)
 #pragma unroll
       for (int i = 0; i < S; ++i)
@@ -506,15 +513,15 @@ cudaError_t split_prepare(int digits) {
 }
 
 cudaError_t split_matrix(const SplitMat &m, const double *src, int digits, cudaStream_t s) {
-  if (digits == 8) k_split_rows<8><<<m.rows, 256, 0, s>>>(src, m.K, m.a, m.ascale);
-  else k_split_rows<7><<<m.rows, 256, 0, s>>>(src, m.K, m.a, m.ascale);
+  if (digits == 8) k_split_rows<8><<<m.rows, 256, 0, s>>>(src, m.K, m.a, m.aexp);
+  else k_split_rows<7><<<m.rows, 256, 0, s>>>(src, m.K, m.a, m.aexp);
   return cudaGetLastError();
 }
 
 template <typename Dc>
 cudaError_t split_rhs(const SplitMat &m, const Dc *z, cudaStream_t s, bool pdl) {
   return launch(k_split_rhs<Dc, split_digits<Dc>()>, dim3((m.K + SPLIT_KB - 1) / SPLIT_KB, (m.T + SPLIT_RT - 1) / SPLIT_RT), 256, 0, s, pdl, z, m.K, m.T, m.b, m.ld,
-                m.ld * m.T, (const unsigned *)m.bmax, m.bscale);
+                m.ld * m.T, (const unsigned *)m.bmax, m.bexp);
 }
 
 template <typename Dc>
@@ -525,7 +532,7 @@ cudaError_t split_product(const SplitMat &m, const SplitOut<Dc> &out, cudaStream
                          (longlong2 *)m.part, n_rt, m.K, m.T, m.nt, m.ks, m.kbps);
   if (e == cudaSuccess)
     e = launch(k_split_sum<Dc, S>, dim3((m.rows + 31) / 32, (m.T + SUM_T - 1) / SUM_T), 32 * SUM_T, 0, s, pdl,
-               (const longlong2 *)m.part, (const float *)m.ascale, (const float *)m.bscale, m.rows, m.T, m.ks, n_rt, out);
+               (const longlong2 *)m.part, (const int *)m.aexp, (const int *)m.bexp, m.rows, m.T, m.ks, n_rt, out);
   return e;
 }
 

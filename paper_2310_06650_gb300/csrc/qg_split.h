@@ -7,7 +7,12 @@
 // splitting of Ozaki, Ogita, Oishi and Rump, Numerical Algorithms 59, 2012).  The digit products with i + j
 // = g share one FP32 accumulator; SPLIT_CHUNK columns and at most S pairs keep it an integer of at most
 // 2^24 (S 128 2^14), so every accumulation is exact, and the accumulators are added up as 64-bit integers.
-// What is dropped are the digit products with i + j >= S.
+// What is dropped are the digit products with i + j >= S.  An output is off by at most
+//   K (S + 1) 2^(4 - 8 S) max|A[row]| max|B[t]|
+// (K columns; the dropped products, and the rounding of both operands to 8 S - 2 bits below the power of two
+// above their largest entry) and the rounding to the result's type: relative to the largest entries, where
+// a sum in FP64 or double-FP32 is relative to sum_k |A B|.  The operands' whole range is covered, the powers of
+// two being kept as exponents; a row or a right-hand side with an infinity or NaN gives NaN.
 #pragma once
 
 #include <cuda.h>
@@ -15,6 +20,8 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+
+#include "qg_internal.h"
 
 namespace qg {
 
@@ -28,6 +35,13 @@ constexpr int SPLIT_SPREAD = 16;  // copies of the running maxima of a right-han
 template <typename Dc>
 constexpr int split_digits() { return sizeof(Dc) == 8 && alignof(Dc) == 8 ? 8 : 7; }
 
+// Key of |v|, increasing with it, whose leading bits are its exponent: what the scales are taken from (a maximum
+// of keys is the same in any order).
+#ifdef __CUDACC__
+__device__ __forceinline__ unsigned split_key(double v) { return (unsigned)__double2hiint(fabs(v)); }
+__device__ __forceinline__ unsigned split_key(df32 v) { return __float_as_uint(__fadd_ru(fabsf(v.hi), fabsf(v.lo))); }
+#endif
+
 // A static matrix in digits, with the tensor maps and the buffers of its right-hand sides.
 struct SplitMat {
   int rows, K, T;           // A is rows x K; T right-hand sides
@@ -36,9 +50,9 @@ struct SplitMat {
   CUtensorMap ta, tb;       // A's tiles as rows of 64; (K, T, S)
   __nv_bfloat16 *a, *b;     // tiles [row tile][K block][S][128][64] (zeroed); [S][T][ld]
   long long ld;             // K rounded up to a multiple of 8
-  float *ascale, *bscale;   // 2^e per row of A and per right-hand side
+  int *aexp, *bexp;         // e per row of A and per right-hand side
   void *part;               // [ks][row tiles][T][128] pairs of 64-bit partial sums
-  unsigned *bmax;           // [SPLIT_SPREAD][T] bits of the largest |B| seen (zeroed before the producer)
+  unsigned *bmax;           // [SPLIT_SPREAD][T] the largest key of B's entries seen (zeroed before the producer)
 };
 
 // Elements of m.a.
