@@ -439,8 +439,8 @@ int qg_mlp_check(qg_mlp *m);
  * library's device arrays (or to a caller's array a handle was given) is checked against the
  * address ranges of those arrays; an access that falls outside all of them reads or writes a
  * dummy word instead, and the first one is recorded.  qg_bounds_report synchronizes the device and
- * returns 1 with that access's source line (of qg_kernels.cu) and address (host pointers, may be
- * NULL), or 0 if none was seen; QG_ERR_UNSUPPORTED in the normal build. */
+ * returns 1 with that access's source line (of qg_kernels.cu; 100,000 + the line for qg_split.cu) and
+ * address (host pointers, may be NULL), or 0 if none was seen; QG_ERR_UNSUPPORTED in the normal build. */
 int qg_bounds_report(int64_t *line, uint64_t *addr);
 
 /* Build identification: major*10000 + minor*100 + patch. */

@@ -36,6 +36,7 @@
 #include <utility>
 #include <vector>
 
+#include "qg_check.h"
 #include "qg_internal.h"
 #include "qg_split.h"
 
@@ -43,35 +44,10 @@ namespace qg {
 
 // ---------------------------------------------------------------------------------------------
 // index-checked build (QG_CHECK_BOUNDS): the build step rewrites every d.<array>[i] of this file
-// as qg_at(d.<array>, i, __LINE__), which checks the element's address against the registered
-// device arrays
+// as qg_at(d.<array>, i, __LINE__); see qg_check.h
 // ---------------------------------------------------------------------------------------------
 
 #ifdef QG_CHECK_BOUNDS
-constexpr int QG_MAX_RANGES = 8192;
-struct QgRange {
-  unsigned long long lo, hi;  // [lo, hi)
-};
-__device__ QgRange g_qg_ranges[QG_MAX_RANGES];  // sorted by lo, disjoint
-__device__ int g_qg_nranges;
-__device__ int g_qg_bad_line;                 // first failing access: its source line (0: none)
-__device__ unsigned long long g_qg_bad_addr;  // and its address
-__device__ __align__(16) unsigned char g_qg_dummy[64];
-
-template <typename T>
-__device__ __forceinline__ T &qg_at(T *p, long long i, int line) {
-  const unsigned long long a = reinterpret_cast<unsigned long long>(p + i);
-  int lo = 0, hi = g_qg_nranges - 1;
-  while (lo <= hi) {  // the last range starting at or below a
-    const int mid = (lo + hi) >> 1;
-    if (g_qg_ranges[mid].lo <= a) lo = mid + 1;
-    else hi = mid - 1;
-  }
-  if (hi >= 0 && a + sizeof(T) <= g_qg_ranges[hi].hi) return p[i];
-  if (atomicCAS(&g_qg_bad_line, 0, line) == 0) g_qg_bad_addr = a;
-  return *reinterpret_cast<T *>(g_qg_dummy);
-}
-
 namespace {
 std::mutex g_ranges_mu;
 std::map<unsigned long long, unsigned long long> g_ranges;  // base -> bytes, every live registration
@@ -81,9 +57,9 @@ void upload_ranges() {
   for (const auto &r : g_ranges) v.push_back({r.first, r.first + r.second});
   if (v.size() > (size_t)QG_MAX_RANGES) v.resize(QG_MAX_RANGES);
   const int n = (int)v.size();
-  cudaDeviceSynchronize();  // no kernel reads the table while it changes (debug build)
-  if (n) cudaMemcpyToSymbol(g_qg_ranges, v.data(), sizeof(QgRange) * n);
-  cudaMemcpyToSymbol(g_qg_nranges, &n, sizeof(int));
+  cudaDeviceSynchronize();  // no kernel reads the tables while they change (debug build)
+  check_upload(v.data(), n);
+  split_check_upload(v.data(), n);
 }
 }  // namespace
 
@@ -109,8 +85,8 @@ int bounds_report(long long *line, unsigned long long *addr) {
   int l = 0;
   unsigned long long a = 0;
   cudaDeviceSynchronize();
-  cudaMemcpyFromSymbol(&l, g_qg_bad_line, sizeof(int));
-  cudaMemcpyFromSymbol(&a, g_qg_bad_addr, sizeof(a));
+  check_first(&l, &a);
+  if (!l) split_check_first(&l, &a);
   if (line) *line = l;
   if (addr) *addr = a;
   return l ? 1 : 0;
@@ -857,7 +833,7 @@ __device__ __forceinline__ void lodf_load4(const void *base, long long idx, int 
     const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162 *>(&u.x), b = *reinterpret_cast<const __nv_bfloat162 *>(&u.y);
     v[0] = __low2float(a); v[1] = __high2float(a); v[2] = __low2float(b); v[3] = __high2float(b);
   } else if (dtype == QG_LODF_BF16X2) {
-    const uint4 u = *reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat162 *>(base) + idx);
+    const uint4 u = QG_AT(reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat162 *>(base) + idx), 0);
     const unsigned w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -865,7 +841,7 @@ __device__ __forceinline__ void lodf_load4(const void *base, long long idx, int 
       v[j] = __low2float(h) + __high2float(h);
     }
   } else {
-    const float4 f = *reinterpret_cast<const float4 *>(static_cast<const float *>(base) + idx);
+    const float4 f = QG_AT(reinterpret_cast<const float4 *>(static_cast<const float *>(base) + idx), 0);
     v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
   }
 }
@@ -1509,19 +1485,19 @@ constexpr size_t hot_smem_bytes() {
 
 // Four consecutive values at p, aligned to the four.
 __device__ __forceinline__ void load4(const float *p, float (&v)[4]) {
-  const float4 q = *reinterpret_cast<const float4 *>(p);
+  const float4 q = QG_AT(reinterpret_cast<const float4 *>(p), 0);
   v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
 }
 __device__ __forceinline__ void load4(const double *p, double (&v)[4]) {
-  const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+  const double2 a = QG_AT(reinterpret_cast<const double2 *>(p), 0), b = QG_AT(reinterpret_cast<const double2 *>(p), 1);
   v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
 __device__ __forceinline__ void store4(float *p, const float (&v)[4]) {
-  *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  QG_AT(reinterpret_cast<float4 *>(p), 0) = make_float4(v[0], v[1], v[2], v[3]);
 }
 __device__ __forceinline__ void store4(double *p, const double (&v)[4]) {
-  reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-  reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+  QG_AT(reinterpret_cast<double2 *>(p), 0) = make_double2(v[0], v[1]);
+  QG_AT(reinterpret_cast<double2 *>(p), 1) = make_double2(v[2], v[3]);
 }
 
 // One element of a hot row: whether it is overloaded, sigma_s(u) (val) and sigma'(u) / s (dd, without the
@@ -2607,9 +2583,9 @@ __device__ __forceinline__ void gbus_products(const Inst &I, const Dc *__restric
 #pragma unroll
     for (int k = 0; k < UN; ++k) {
       const int m = m0 + k * 32 + lane;
-      av[k] = m < I.M ? A[m] : DcOps<Dc>::zero();
+      av[k] = m < I.M ? QG_AT(A, m) : DcOps<Dc>::zero();
 #pragma unroll
-      for (int i = 0; i < NT; ++i) gv[i][k] = m < I.M && i < nt ? gf[(long long)i * I.M + m] : Real(0);
+      for (int i = 0; i < NT; ++i) gv[i][k] = m < I.M && i < nt ? QG_AT(gf, (long long)i * I.M + m) : Real(0);
     }
 #pragma unroll
     for (int i = 0; i < NT; ++i)
@@ -2872,11 +2848,11 @@ __global__ void __launch_bounds__(NTHR) k_sp_fwd(const __grid_constant__ Dev<Rea
         unsigned *mx = d.sp_bmax + ((ADJ ? SPLIT_SPREAD : 0) + row % SPLIT_SPREAD) * T;
         if (ta < T) {
           z[ta] = z0 = DcOps<Dc>::add(b[ta], z0);
-          atomicMax(mx + ta, split_key(z0));
+          atomicMax(&QG_AT(mx, ta), split_key(z0));
         }
         if (tb < T) {
           z[tb] = z1 = DcOps<Dc>::add(b[tb], z1);
-          atomicMax(mx + tb, split_key(z1));
+          atomicMax(&QG_AT(mx, tb), split_key(z1));
         }
       }
       __syncthreads();

@@ -16,6 +16,7 @@
 #include <cmath>
 #include <mutex>
 
+#include "qg_check.h"
 #include "qg_internal.h"
 #include "qg_split.h"
 #include "qg_split_feed.h"
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1)
 #pragma unroll
       for (int c = 0; c < SPLIT_NT / 2; ++c)
         if (c < hc && p * nt + half * hc + c < T)
-          dst[c * SPLIT_ROWS] = ok ? make_longlong2(hi[c], lo[c]) : make_longlong2(SPLIT_LOST, 0);
+          QG_AT(dst, c * SPLIT_ROWS) = ok ? make_longlong2(hi[c], lo[c]) : make_longlong2(SPLIT_LOST, 0);
     }
   }
   __syncwarp();
@@ -330,16 +331,16 @@ __global__ void __launch_bounds__(32 * SUM_T) k_split_sum(const longlong2 *__res
   __shared__ Dc s_v[32][SUM_T + 1];
   const int r0 = blockIdx.x * 32, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int t0 = blockIdx.y * SUM_T, tn = min(SUM_T, T - t0);
-  const int ea = aexp[min(r0 + lane, rows - 1)];
+  const int ea = QG_AT(aexp, min(r0 + lane, rows - 1));
   wait_grid();
   const int t = min(t0 + wid, T - 1);
   const longlong2 *src = part + ((long long)(r0 / SPLIT_ROWS) * T + t) * SPLIT_ROWS + r0 % SPLIT_ROWS + lane;
-  const int eb = bexp[t];
+  const int eb = QG_AT(bexp, t);
   long long hi = 0, lo = 0;
   bool lost = ea == SPLIT_NONFINITE || eb == SPLIT_NONFINITE;
 #pragma unroll 8
   for (int q = 0; q < ks; ++q) {
-    const longlong2 v = src[(long long)q * n_rt * T * SPLIT_ROWS];
+    const longlong2 v = QG_AT(src, (long long)q * n_rt * T * SPLIT_ROWS);
     lost |= v.x == SPLIT_LOST;
     hi += v.x;
     lo += v.y;
@@ -349,11 +350,11 @@ __global__ void __launch_bounds__(32 * SUM_T) k_split_sum(const longlong2 *__res
   const int r = threadIdx.x / SUM_T, tt = threadIdx.x % SUM_T, pos = out.pos0 + r0 + r;
   if (r0 + r >= rows || tt >= tn) return;
   const Dc v = s_v[r][tt];
-  out.u[(long long)pos * T + t0 + tt] = v;
-  out.th[(long long)pos * T + t0 + tt] = v;  // forward: the angles; adjoint: eta (transformer gradients)
+  QG_AT(out.u, (long long)pos * T + t0 + tt) = v;
+  QG_AT(out.th, (long long)pos * T + t0 + tt) = v;  // forward: the angles; adjoint: eta (transformer gradients)
   if (out.pos_gb) {
-    const int gb = out.pos_gb[pos];
-    if (gb >= 0) out.gip[(long long)(t0 + tt) * out.gi_ld + gb] = v;
+    const int gb = QG_AT(out.pos_gb, pos);
+    if (gb >= 0) QG_AT(out.gip, (long long)(t0 + tt) * out.gi_ld + gb) = v;
   }
 }
 
@@ -397,23 +398,23 @@ __global__ void __launch_bounds__(256) k_split_rows(const double *__restrict__ s
   __shared__ int s_e;
   const double *row = src + (long long)blockIdx.x * K;
   unsigned mx = 0;
-  for (int k = threadIdx.x; k < K; k += 256) mx = max(mx, split_key(row[k]));
+  for (int k = threadIdx.x; k < K; k += 256) mx = max(mx, split_key(QG_AT(row, k)));
   mx = __reduce_max_sync(0xffffffffu, mx);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) mx = max(mx, red[w]);
     s_e = split_exp(mx, 0.0);
-    aexp[blockIdx.x] = s_e;
+    QG_AT(aexp, blockIdx.x) = s_e;
   }
   __syncthreads();
   const int rt = blockIdx.x / SPLIT_ROWS, r = blockIdx.x % SPLIT_ROWS, nkb = (K + SPLIT_KB - 1) / SPLIT_KB;
   for (int k = threadIdx.x; k < K; k += 256) {
     float q[S];
-    digits<S>(s_e != SPLIT_NONFINITE ? fixed_point(row[k], 8 * S - 2 - s_e) : 0ll, q);
+    digits<S>(s_e != SPLIT_NONFINITE ? fixed_point(QG_AT(row, k), 8 * S - 2 - s_e) : 0ll, q);
     __nv_bfloat16 *dst = a + (((long long)(rt * nkb + k / SPLIT_KB) * S) * SPLIT_ROWS + r) * SPLIT_KB + k % SPLIT_KB;
 #pragma unroll
-    for (int i = 0; i < S; ++i) dst[(long long)i * SPLIT_ROWS * SPLIT_KB] = __float2bfloat16_rn(q[i]);
+    for (int i = 0; i < S; ++i) QG_AT(dst, (long long)i * SPLIT_ROWS * SPLIT_KB) = __float2bfloat16_rn(q[i]);
   }
 }
 
@@ -429,14 +430,14 @@ __global__ void __launch_bounds__(256) k_split_rhs(const Dc *__restrict__ z, int
   const int t0 = blockIdx.y * SPLIT_RT, tn = min(SPLIT_RT, T - t0);
   for (int e = threadIdx.x; e < kn * tn; e += 256) {
     const int k = e / tn, t = e - k * tn;
-    s_z[k][t] = z[(long long)(k0 + k) * T + t0 + t];
+    s_z[k][t] = QG_AT(z, (long long)(k0 + k) * T + t0 + t);
   }
   if ((int)threadIdx.x < tn) {
     unsigned m = 0;
 #pragma unroll
-    for (int q = 0; q < SPLIT_SPREAD; ++q) m = max(m, bmax[q * T + t0 + threadIdx.x]);
+    for (int q = 0; q < SPLIT_SPREAD; ++q) m = max(m, QG_AT(bmax, q * T + t0 + threadIdx.x));
     s_e[threadIdx.x] = split_exp(m, Dc{});
-    if (blockIdx.x == 0) bexp[t0 + threadIdx.x] = s_e[threadIdx.x];
+    if (blockIdx.x == 0) QG_AT(bexp, t0 + threadIdx.x) = s_e[threadIdx.x];
   }
   __syncthreads();
   for (int t = wid; t < tn; t += 8) {  // lanes: pairs of consecutive k, one 128-byte line per (digit, t)
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(256) k_split_rhs(const Dc *__restrict__ z, int
     if (k0 + k < (int)ld)
 #pragma unroll
       for (int i = 0; i < S; ++i)
-        *reinterpret_cast<__nv_bfloat162 *>(b + i * slice + (long long)(t0 + t) * ld + k0 + k) =
+        QG_AT(reinterpret_cast<__nv_bfloat162 *>(b + i * slice + (long long)(t0 + t) * ld + k0 + k), 0) =
             __floats2bfloat162_rn(q0[i], q1[i]);
   }
 }
@@ -505,6 +506,14 @@ bool split_maps(SplitMat &m, int digits) {
   const cuuint32_t bb[3] = {SPLIT_KB, (cuuint32_t)m.nt, (cuuint32_t)digits};
   return encode(&m.ta, m.a, 2, da, sa, ba) && encode(&m.tb, m.b, 3, db, sb, bb);
 }
+
+#ifdef QG_CHECK_BOUNDS
+void split_check_upload(const QgRange *v, int n) { check_upload(v, n); }
+void split_check_first(int *line, unsigned long long *addr) {
+  check_first(line, addr);
+  if (*line) *line += 100000;
+}
+#endif
 
 cudaError_t split_prepare(int digits) {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;

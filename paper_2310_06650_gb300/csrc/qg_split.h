@@ -82,6 +82,13 @@ struct SplitOut {
   long long gi_ld;
 };
 
+#ifdef QG_CHECK_BOUNDS
+// The index checks of qg_split.cu (qg_check.h): its table, and its first miss as 100,000 + the source line.
+struct QgRange;
+void split_check_upload(const QgRange *v, int n);
+void split_check_first(int *line, unsigned long long *addr);
+#endif
+
 template <typename Dc>
 cudaError_t split_product(const SplitMat &m, const SplitOut<Dc> &out, cudaStream_t s, bool pdl);
 
