@@ -138,6 +138,8 @@ typedef struct {
                         * QG_DC_SPARSE: the sparse factor Yhat = L diag(D_S, S) L^T with a dense
                         *   tail, two gathers and one dense product per solve, for the base flows
                         *   (Eq. Yb_solve) and the adjoint (Eq. 2nd_lin_sys); no PTDF is formed.
+                        *   Of device memory, an entry of the tail's inverse (n_T x n_T) takes 16 bytes
+                        *   on the FP64 path, 14 on the mixed one, and 8 more while it is created.
                         *   One instance per handle (QG_ERR_UNSUPPORTED otherwise);
                         * QG_DC_AUTO (0, the default): sparse for a single instance of more
                         *   than 4096 buses, dense otherwise.
@@ -199,7 +201,9 @@ int qg_set_stream(qg_ctx *h, void *stream);
 /* One full evaluation (Eq. grads): obj[b] = Phi_b(x) for every instance b
  * (device, n_inst doubles) and g = grad Phi(x) (device, qg_num_vars elements),
  * covering every period and every contingency (Alg. 2 with K_t = all, zeta = 0).
- * g may be NULL (objective only).  x is not modified. */
+ * g may be NULL (objective only).  x is not modified, unless g or obj overlaps it.  The stage kernels
+ * write g and obj where these are aligned memory of the handle's GPU apart from x and from each other;
+ * other arrays (of another GPU, managed, unaligned, overlapping) take a copy after them. */
 int qg_eval_grad(qg_ctx *h, const void *x, double *obj, void *g);
 
 /* qg_eval_grad without any allocation, for callers that cannot call cudaMalloc at this point
@@ -207,12 +211,13 @@ int qg_eval_grad(qg_ctx *h, const void *x, double *obj, void *g);
  * whose memory pool is already sized and frozen).  The paper has no counterpart: it is an
  * interface addition.  The handle's set-up data (made by qg_create) is reused; every
  * per-evaluation work buffer comes from one file-scope static device array of 32 MiB (16 MiB of work
- * buffers, and at most as much for the hot rows' sums of stage 2) that every GPU loading the library
+ * buffers, and at most as much for the hot rows' sums and flags of stage 2 and, on the FP64 path, the
+ * sines and cosines of the angles across the branches) that every GPU loading the library
  * holds from load until the process exits.  The caller passes the inputs
  * and outputs: x (device, qg_num_vars elements), obj (device, n_inst doubles) and g (device,
  * qg_num_vars elements, required).  Results equal those of qg_eval_grad.
- *  - Handles whose work buffers need more than 16 MiB without those sums (e.g. large batches) are rejected with
- *    QG_ERR_UNSUPPORTED and a message giving the size needed; so are handles on the sparse DC
+ *  - Handles whose work buffers need more than 16 MiB without the second half (e.g. large batches) are
+ *    rejected with QG_ERR_UNSUPPORTED and a message giving the size needed; so are handles on the sparse DC
  *    solver (QG_DC_SPARSE), whose solve buffers are not carved from the array, and handles with
  *    contingency screening (0 < ctg_frac < 1), whose compacted line-outage block is not either.
  *  - The first call on a device looks up the array's device address (cudaGetSymbolAddress); make
@@ -412,7 +417,8 @@ void qg_mlp_destroy(qg_mlp *m);
 int64_t qg_mlp_num_params(const qg_mlp *m);
 int qg_mlp_set_stream(qg_mlp *m, void *stream);
 
-/* Inference: y = MLP(x) for `batch` rows (batch <= max_batch). */
+/* Inference: y = MLP(x) for `batch` rows (batch <= max_batch).  y that is not memory of the network's GPU
+ * aligned to floats takes a copy. */
 int qg_mlp_forward(qg_mlp *m, const float *x, int32_t batch, float *y);
 
 /* One training step on the mean squared error mean((Y - target)^2): forward, backward, and (if

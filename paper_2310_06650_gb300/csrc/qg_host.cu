@@ -580,8 +580,8 @@ std::vector<df32> to_dc<df32>(const std::vector<double> &v) {
   return o;
 }
 
-// A stage holds at most three spans per instance (stage 1: DC flows, branches, zones) plus one
-// for the sparse solver's adjoint right-hand side, so MAXB instances never overflow the table.
+// A stage holds at most four spans per instance (stage 1: DC flows, branches, bus balances, zones) plus
+// one for the sparse solver's adjoint right-hand side, so MAXB instances never overflow the table.
 static_assert(MAXSPAN >= 4 * MAXB + 1, "span table too small for MAXB instances");
 
 void add_span(Spans &S, int per_t, int nt, int inst, int role) {
@@ -780,11 +780,11 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
   for (int b = 0; b < B; ++b) add_span(P.s3, I[b].fold_nb, 1, b, R_OBJ);
   for (int b = 0; b < B; ++b) add_span(P.s3, I[b].n_sb, I[b].T, b, R_BRANCH);
   // adjoint DC products and devices.  Dense mode: one warp per (period, generator bus or transformer
-  // column) in stage 4 computes the adjoint product; on the mixed path the warp also updates the
-  // devices at the bus (stage 4 is the last stage); the FP64 path leaves the devices to stage 5 blocks
-  // of 32 (period, device) pairs, so that each warp's FP64 instructions serve 32 devices.  Sparse
-  // mode: the adjoint solve follows stage 4, and stage 5 updates the devices (FP64 path: one warp of
-  // pairs per block; mixed path: a full block of pairs), then the transformers.
+  // column) in stage 4 computes the adjoint product, on large plans one per (GB_TC periods, column) in
+  // k_gbus; on small plans of the mixed path the warp also updates the devices at the bus (stage 4 is the
+  // last stage), otherwise stage 5 does.  Sparse mode: the adjoint solve follows stage 4.  Stage 5 takes a
+  // full block of (period, device) pairs on the mixed path, 8 or 64 pairs of four lanes each on the FP64
+  // path, then the transformers.
   const bool fuse = !P.sp && small_mixed;
   P.tab.fuse = fuse ? 1 : 0;
   int gen_slot = 0;
@@ -805,8 +805,8 @@ int build_plan(qg_ctx *h, std::vector<int> &slot_map, const Knobs &kn) {
     add_span(P.s4, ceil_div(H0.n - 1, 32), ceil_div(H0.T, DCF_TC), 0, R_SDCA);
   if (!fuse) {
     // FP64: one warp of pairs per block (GB300's FP64 pipe costs as much for a warp with one active
-    // lane as for a full one), 8 pairs of four lanes each; whole blocks
-    // where there are several per SM of them (day-ahead grid: 18,000 blocks of one warp took 351 us)
+    // lane as for a full one), 8 pairs of four lanes each; whole blocks of 64 pairs where there are several
+    // per SM of them (day-ahead grid: 18,000 blocks of one warp took 351 us, whole blocks 126)
     for (int b = 0; b < B; ++b) {
       const bool big = (long long)I[b].T * I[b].G > 8 * 152 * 64;
       const int gen_pb = h->opt.precision == QG_FP64 ? (big ? NTHR / 4 : 8) : NTHR;
@@ -896,7 +896,6 @@ int upload_selection(qg_ctx *h, int b) {
   return QG_OK;
 }
 
-// Build every device array of one precision flavour.
 void dfree(qg_ctx *h, const void *p);
 
 // S^-1 of the dense tail in digits for the tensor cores (qg_split.h), its buffers and tensor maps.
@@ -935,6 +934,7 @@ int build_tail(qg_ctx *h, Dev<Real, Dc> &d, const HostInst &H) {
   return QG_OK;
 }
 
+// Build every device array of one precision flavour.
 template <typename Real, typename Dc>
 int build_device(qg_ctx *h, Dev<Real, Dc> &d, const std::vector<int> &slot_map) {
   const int B = h->n_inst;
@@ -1629,7 +1629,8 @@ int eval_noalloc(qg_ctx *h, Dev<Real, Dc> d, const void *x, double *obj, void *g
   d.trace_len = 0;
   bounds_register(obj, sizeof(double) * h->n_inst);  // the caller's arrays (index-checked builds)
   bounds_register(g, sizeof(Real) * h->n_x);
-  // the closing kernel reads and rewrites the step counter (the rest is fully written before it is read)
+  // the closing kernel reads and rewrites the step counter (the rest is written before it is used; what is
+  // read without having been written, row partials of tiles without a flag, is not selected)
   CUDA_TRY(h, cudaMemsetAsync(d.step, 0, sizeof(long long), h->stream));
   cudaError_t e = launch_eval<Real, Dc>(d, h->plan, x, false, true, h->stream, nullptr);
   if (e != cudaSuccess) return fail(h, QG_ERR_CUDA, std::string("evaluation launch: ") + cudaGetErrorString(e));

@@ -1803,6 +1803,7 @@ template <typename Real, typename Dc, int SPLIT, bool HOT, int NI>
 __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __grid_constant__ Dev<Real, Dc> d,
                                              const __grid_constant__ InstTabT<NI> tab, const __grid_constant__ SpansT<NI> S,
                                              const Real *__restrict__ x) {
+  static_assert(!HOT || SPLIT == 1, "the warp's sums over hot rows take one branch per thread");
   const Where w = locate(S);
   const Inst &I = tab.I[NI == 1 || tab.n_inst == 1 ? 0 : w.inst];  // one instance: no wait on the span search
   if (w.role == R_OBJ) {  // whole block
@@ -1875,9 +1876,8 @@ __global__ void __launch_bounds__(NTHR, sizeof(Real) == 4 ? 3 : 2) k_s3(const __
           if (kt % SPLIT == q && d.pmf[I.pf0 + ((long long)kt * I.T + t) * I.n_mt + (j >> 6)]) set |= 1u << (kt - k0);
       }
       if (hot) {
-        set = 0;
-        for (int kt = k0; kt < min(I.n_kt, k0 + 32); kt += HOT_BK / CT_BK)
-          if (kt % SPLIT == q) set |= 1u << (kt - k0);
+        set = 0;  // (one thread per branch: HOT comes with SPLIT = 1)
+        for (int kt = k0; kt < min(I.n_kt, k0 + 32); kt += HOT_BK / CT_BK) set |= 1u << (kt - k0);
       }
       for (set = on ? set : 0; set; set &= set - 1) {
         const long long pq = I.pm0 + ((long long)(k0 + __ffs(set) - 1) * I.T + t) * I.M + j;
